@@ -1,0 +1,142 @@
+"""The kernels at the sizes where their work split can go wrong: lattices that
+do not fill a warp, a block or a group of blocks, odd snapshot strides, boxes
+whose cell edge rounds, tetrahedra of zero volume, and the smallest and
+odd-sized grids, against FP64 (numpy or the oracle).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from lt_inputs import ZeldovichField, fp16_offsets
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TETS = np.array([[1, 0, 2, 4], [3, 1, 2, 4], [3, 5, 1, 4], [3, 6, 5, 4], [3, 2, 6, 4], [3, 7, 5, 6]])
+
+
+@pytest.fixture(scope="module")
+def R():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1208_3206_gb300.render import Renderer
+    return Renderer()
+
+
+def lattice(N, lam, seed, box=1.0):
+    if N < 4:  # too small for the generator's spectrum
+        rng = np.random.default_rng(seed)
+        d = rng.uniform(-0.2, 0.2, (N ** 3, 3)) * lam / N
+    else:
+        d = ZeldovichField.generate(N, -2.0, 0.375 * N, seed).displacement(lam)
+    return d  # in units of a unit box, [N^3][3]
+
+
+def wrapped(d, N, box):
+    i = np.arange(N ** 3)
+    q = np.stack([i % N, (i // N) % N, i // (N * N)], axis=1) * (box / N)
+    x = np.mod(q + d * box, box).astype(np.float32)
+    out = np.zeros((N ** 3, 4), dtype=np.float32)
+    out[:, :3] = np.where(x >= np.float32(box), np.float32(0), x)
+    return out
+
+
+def volumes(disp, N, h):
+    """Signed volumes [6 N^3] from FP64 displacements and the cell edge h."""
+    c = np.arange(N ** 3)
+    i, j, k = c % N, (c // N) % N, c // (N * N)
+    corner = []
+    for n in range(8):
+        a, b, e = n & 1, (n >> 1) & 1, n >> 2
+        idx = (i + a) % N + N * ((j + b) % N + N * ((k + e) % N))
+        corner.append(disp[idx] + np.array([a, b, e]) * h)
+    v = np.stack(corner, axis=1)[:, TETS]  # [N^3][6][4][3]
+    e = v[:, :, 1:] - v[:, :, :1]
+    return (np.einsum("tsa,tsa->ts", e[:, :, 0], np.cross(e[:, :, 1], e[:, :, 2])) / 6.0).reshape(-1)
+
+
+def unwrapped(pos, N, box):
+    i = np.arange(N ** 3)
+    q = np.stack([i % N, (i // N) % N, i // (N * N)], axis=1) * (box / N)
+    d = pos[:, :3].astype(np.float64) - q
+    return d - box * np.round(d / box)
+
+
+@pytest.mark.parametrize("N,box,half,snaps", [(1, 1.0, False, 1), (2, 1.0, False, 3), (3, 1.0, False, 2), (7, 100.0, False, 3),
+                                              (8, 1.0, True, 1), (16, 1.0, False, 2), (33, 1.0, False, 1),
+                                              (33, 40.0, True, 2), (64, 1.0, False, 1)])
+def test_densities(R, N, box, half, snaps):
+    """Densities of every tetrahedron. The FP32 determinant of a volume above
+    0.1 h^3 is off by a few 2^-24 of the product of its edges (here below
+    4^3 h^3): 1e-4 relative. Smaller volumes come from exact edges: FP32's
+    rounding of the density (2^-24) and what h = box / N, a rounded number
+    off a power of two, moves the edges that wrap by (2^-24 N h each). Both
+    sides' FP64 determinants round by 64 h^3 2^-49, which hides the density's
+    last bit below 2^-20 h^3; whether a volume is zero is compared where the
+    products are exact in FP64 (11-bit offsets)."""
+    pos, ref, zero = [], [], 0
+    hf = np.float32(box) / np.float32(N)
+    for s in range(snaps):
+        d = lattice(N, 2.5, 11 + s)
+        # tetrahedra of exactly zero volume (N >= 8): a particle on its neighbour
+        if half:
+            p = fp16_offsets(d, N)
+            if N >= 8:
+                p[6] = (0.25, -0.5, 0.125, 0)
+                p[5] = (1.25, -0.5, 0.125, 0)
+            disp = (p[:, :3].astype(np.float32) * hf).astype(np.float64)
+            h = float(hf)
+        else:
+            p = wrapped(d, N, box)
+            if N >= 8:
+                p[5] = p[6]
+            disp, h = unwrapped(p, N, box), box / N
+        v = volumes(disp, N, h)
+        pos.append(p)
+        ref.append(v)
+        zero += int((v == 0).sum())
+    pos, v = np.stack(pos), np.stack(ref)
+    out = torch.full((snaps, 6 * N ** 3), -1.0, dtype=torch.float32, device="cuda")
+    R.build_tets(torch.from_numpy(pos).cuda(), N, box, rho_out=out)
+    st = R.get_stats()
+    got = out.cpu().numpy().astype(np.float64)
+    with np.errstate(divide="ignore"):
+        rho = 1.0 / (6.0 * N ** 3) / np.abs(v)
+    h3 = (box / N) ** 3
+    small = np.abs(v) < 0.0999 * h3
+    exact = (N & (N - 1)) == 0
+    tol = np.where(small, 2.0 ** -23, 1e-4) + (0.0 if exact else 1.0) * 64 * 2.0 ** -24 * N * h3 / np.maximum(np.abs(v), 1e-300)
+    ok = np.abs(v) > (2.0 ** -20 if exact else 1e-3) * h3
+    assert np.all(np.abs(got - rho)[ok] <= (tol * rho)[ok])
+    if exact and half:
+        assert zero > 0
+        assert st["degenerate"] == zero
+        assert np.all(got[v == 0] == 0)
+        assert st["inverted"] == int((v > 0).sum())
+
+
+@pytest.mark.parametrize("N,n,z0,half", [(1, 3, 0.3, False), (2, 1, 0.4, False), (5, 33, -0.21, False), (9, 31, 7.77, False),
+                                         (16, 200, 0.999, True), (11, 64, 0.013, False)])
+@pytest.mark.parametrize("weight", ["streams", "density"])
+def test_slices(R, N, n, z0, half, weight):
+    """Slice points against the oracle: counts equal, densities to 1e-5 (FP64
+    volumes on both sides, sums of 2^-28 of the mean and FP32's rounding)."""
+    d = lattice(N, 1.7, 5)
+    if half:
+        p = fp16_offsets(d, N)
+        i = np.arange(N ** 3)
+        q = np.stack([i % N, (i // N) % N, i // (N * N)], axis=1) / N
+        ref_pos = np.mod(q + p[:, :3].astype(np.float64) / N, 1.0)
+    else:
+        p = ref_pos = wrapped(d, N, 1.0)
+    R.build_tets(torch.from_numpy(p).cuda(), N)
+    got = R.slice(n, z0, weight).cpu().numpy().astype(np.float64).ravel()
+    R.sync()
+    a = (np.arange(n) + 0.5) / n
+    X, Y = np.meshgrid(a, a)
+    pts = np.stack([X.ravel(), Y.ravel(), np.full(n * n, z0 - np.floor(z0))], axis=1)
+    ref = oracle.point_density(ref_pos, N, pts, weight)
+    if weight == "streams":
+        assert np.array_equal(got, ref)
+    else:
+        assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
