@@ -72,7 +72,8 @@ cudaError_t launch_slice(const Lattice& L, int snapshot, int n, int weight, doub
 // the far cubes (cube_far) are drawn.
 cudaError_t launch_centroids(const Lattice& L, const FrameDev* d_frame, int W, int H, double m_tet, double unit,
                              unsigned long long* d_acc, float* d_out, bool add, DevCounters* ctr, cudaStream_t s);
-// 64-bit fixed-point sums (units of `unit`) to float, overwriting or adding to d_out.
+// 64-bit fixed-point sums (units of `unit`) to float, overwriting or adding to
+// d_out (the last step of every kernel that sums in global memory).
 cudaError_t launch_fixed_finalize(const unsigned long long* d_acc, long long np, double unit, bool add, float* d_out,
                                   cudaStream_t s);
 

@@ -200,12 +200,6 @@ __global__ void __launch_bounds__(kResampleThreads) k_resample(ResampleArgs a) {
   }
 }
 
-__global__ void k_resample_finalize(const unsigned long long* __restrict__ acc, long long cells, double unit,
-                                    float* __restrict__ out) {
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < cells; p += (long long)gridDim.x * blockDim.x)
-    out[p] = (float)((double)acc[p] * unit);
-}
-
 cudaError_t launch_resample(const Lattice& L, const FrameDev* d_frame, long long n_tiles, int tile,
                             const unsigned long long* d_off, const unsigned* d_list, unsigned long long list_cap, int n,
                             int weight, double m_tet, double unit, unsigned long long* d_acc, float* d_out,
@@ -230,10 +224,7 @@ cudaError_t launch_resample(const Lattice& L, const FrameDev* d_frame, long long
   k_resample<<<(unsigned)n_tiles, kResampleThreads, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  long long blocks = (cells + 255) / 256;
-  if (blocks > 152LL * 32) blocks = 152LL * 32;
-  k_resample_finalize<<<(unsigned)blocks, 256, 0, s>>>(d_acc, cells, unit, d_out);
-  return cudaGetLastError();
+  return launch_fixed_finalize(d_acc, cells, unit, false, d_out, s);
 }
 
 }  // namespace lt
