@@ -101,7 +101,8 @@ typedef struct {
 
 /* Tuning knobs (lt_autotune fills them; zero fields take defaults). */
 typedef struct {
-  int tile;           /* screen tile edge in pixels: 8, 16, 32 or 64 (default 16) */
+  int tile;           /* screen tile edge in pixels: 8, 16, 32 or 64 (default 16; where it is left 0, the
+                         raster takes 32 for FP32 frames of more than 2^20 pixels: lt_stats.tile) */
   int raster_threads; /* threads per raster CTA: 64..256, multiple of 32 (default 256) */
   int ctas_per_sm;    /* persistent raster CTAs per SM (default: occupancy limit) */
   int frac_bits;      /* fixed-point fraction bits relative to the mean column density sigma, 8..62
@@ -127,8 +128,8 @@ typedef struct {
   long long area_pairs;         /* lt_render_area: (tetrahedron, pixel) pairs walked, last call */
   long long area_fp64_pairs;    /* lt_render_area: of them, clipped in FP64 (hulls under 1/20 pixel wide, or an
                                    apex within 1e-3 pixel of a hull edge) */
-  long long exact_tile_max;     /* most ill-conditioned fragments found in one tile since lt_create (the queue
-                                   holds 64 per pixel of a tile) */
+  long long exact_tile_max;     /* most ill-conditioned fragments found in one work item (a tile, or a part of a long
+                                   tile's list) since lt_create (the queue holds 64 per pixel of a tile) */
   int n_frames;              /* frames of the last lt_project_bin */
   int tile;                  /* tile edge in use */
   int graph_kernels;         /* kernel nodes in the graph of the last lt_graph_build */
@@ -175,8 +176,8 @@ lt_status lt_build_tets(lt_ctx* ctx, const void* d_pos, int pos_fmt, int N, floa
  * frame_snapshot[f] (host array, NULL = snapshot 0 for every frame), bins
  * every lattice cube into the screen tiles its projected bounding box
  * overlaps: warp-aggregated per-tile counts, a device exclusive scan, then a
- * scatter of cube ids into per-tile lists. Also orders the (frame, tile) work
- * items by descending list length for the raster pass.
+ * scatter of cube ids into per-tile lists. Also splits long lists and orders
+ * the (frame, tile) work items by descending length for the raster pass.
  * Outside stream capture the call synchronises once to size the lists
  * (growing the context's buffers as needed). Inside stream capture it uses
  * the reserved capacity and latches LT_ERR_CAPACITY if it is exceeded.

@@ -20,6 +20,7 @@ struct lt_ctx {
   int device = 0;
   int num_sms = 1;
   lt_config cfg{};
+  bool tile_auto = true;  // the caller left the tile edge to the library (see raster_tile)
   // registered lattice
   bool have_lattice = false;
   Lattice L{};
@@ -42,7 +43,12 @@ struct lt_ctx {
   unsigned* d_cursor = nullptr;
   unsigned long long* d_off = nullptr;
   unsigned long long* d_work = nullptr;
+  size_t work_cap = 0;
   double* d_mass_tile = nullptr;
+  unsigned long long* d_slot_acc = nullptr;  // sums of the tiles rastered in several items (zero between renders)
+  size_t slot_acc_cap = 0;
+  unsigned* d_slot_done = nullptr;
+  size_t slot_done_cap = 0;
   unsigned long long* d_xq = nullptr;  // exact-evaluation queues of the raster CTAs
   size_t xq_cap = 0;
   unsigned long long* d_scan_tmp = nullptr;
@@ -301,8 +307,13 @@ bool make_frame(const lt_camera& c, const lt_ctx* ctx, int snapshot, int tile, i
     F.lod[1] = c.lo[1];
     F.pxd[0] = ((double)c.hi[0] - c.lo[0]) / c.W;
     F.pxd[1] = ((double)c.hi[1] - c.lo[1]) / c.H;
+  } else {
+    F.pxd[0] = 1.0 / c.W;
+    F.pxd[1] = 1.0 / c.H;
   }
   F.m_tet = m;
+  F.exact_scale = 6.0 * m / F.unit;
+  F.scale = lt::fixed_scale(F.unit);
   F.sigma_units = (float)scale_bits;
   F.near_r2 = c.near_radius > 0.0 ? c.near_radius * c.near_radius : 0.0;
   return true;
@@ -345,6 +356,23 @@ lt_status prepare_frames(lt_ctx* ctx, const lt_camera* cams, int n_frames, const
   return LT_OK;
 }
 
+// Raster work items beyond one per tile (see work_chunk): a number of the
+// context, not of the launch, so that the slots allocated with the tiles and
+// the lists binned with them always fit.
+unsigned work_target(const lt_ctx* ctx) {
+  return (unsigned)ctx->num_sms * 2u * lt::kItemsPerCta;
+}
+
+// A buffer that has to read zero at its first use.
+template <typename T>
+lt_status grow_zeroed(lt_ctx* ctx, T** p, size_t* cap, size_t n, cudaStream_t s) {
+  if (*cap >= n && *p) return LT_OK;
+  lt_status st = grow_c(ctx, p, cap, n);
+  if (st != LT_OK) return st;
+  LT_CUDA(cudaMemsetAsync(*p, 0, *cap * sizeof(T), s));
+  return LT_OK;
+}
+
 // Launches of the bin pass after the frames are on the device.
 lt_status bin_launches(lt_ctx* ctx, cudaStream_t s, bool allow_sync) {
   const long long n = ctx->n_tiles;
@@ -366,11 +394,12 @@ lt_status bin_launches(lt_ctx* ctx, cudaStream_t s, bool allow_sync) {
   LT_CUDA(cudaMemsetAsync(ctx->d_cursor, 0, sizeof(unsigned) * n, s));
   LT_CUDA(lt::launch_bin_scatter(ctx->L, ctx->d_frames, ctx->n_frames, ctx->d_off, ctx->d_cursor, ctx->d_list,
                                  ctx->list_cap, ctx->d_desc, ctx->d_ctr, s));
-  LT_CUDA(lt::launch_worklist(ctx->d_off, n, ctx->d_hist, ctx->d_work, s));
+  // (the cursors are spent: their array takes the tiles' slots)
+  LT_CUDA(lt::launch_worklist(ctx->d_off, n, work_target(ctx), ctx->d_hist, ctx->d_work, ctx->d_cursor, s));
   return LT_OK;
 }
 
-lt_status ensure_tiles(lt_ctx* ctx, long long n) {
+lt_status ensure_tiles(lt_ctx* ctx, long long n, int tile, cudaStream_t s) {
   lt_status st;
   size_t c;
   if ((size_t)n > ctx->tiles_cap) {
@@ -381,24 +410,44 @@ lt_status ensure_tiles(lt_ctx* ctx, long long n) {
     c = 0;
     if ((st = grow_c(ctx, &ctx->d_off, &c, (size_t)n + 1)) != LT_OK) return st;
     c = 0;
-    if ((st = grow_c(ctx, &ctx->d_work, &c, (size_t)n)) != LT_OK) return st;
-    c = 0;
     if ((st = grow_c(ctx, &ctx->d_mass_tile, &c, (size_t)n)) != LT_OK) return st;
     ctx->tiles_cap = (size_t)n;
   }
+  const size_t target = work_target(ctx);
+  if ((st = grow_c(ctx, &ctx->d_work, &ctx->work_cap, (size_t)n + target)) != LT_OK) return st;
+  if ((st = grow_zeroed(ctx, &ctx->d_slot_acc, &ctx->slot_acc_cap, target * tile * tile, s)) != LT_OK)
+    return st;
+  if ((st = grow_zeroed(ctx, &ctx->d_slot_done, &ctx->slot_done_cap, target, s)) != LT_OK) return st;
   const size_t words = lt::scan_tmp_words(n);
   if ((st = grow_c(ctx, &ctx->d_scan_tmp, &ctx->scan_tmp_cap, words)) != LT_OK) return st;
-  const size_t xq = (size_t)ctx->num_sms * lt::kRasterMaxCtasPerSm * lt::kExactQueuePerPixel * ctx->cfg.tile *
-                    ctx->cfg.tile;
+  const size_t xq = (size_t)ctx->num_sms * lt::kRasterMaxCtasPerSm * lt::kExactQueuePerPixel * tile * tile;
   if ((st = grow_c(ctx, &ctx->d_xq, &ctx->xq_cap, xq)) != LT_OK) return st;
   return LT_OK;
 }
 
+// Tile edge of the raster where the caller left it open: 32 pixels for frames
+// of more than 2^20. A tetrahedron is set up once for every tile it touches,
+// about (1 + s / T)^2 times for a cell of s pixels, and a span ends at the
+// tile's edge, so larger tiles do less work; but only tiles up to 32 pixels
+// leave shared memory for three CTAs per SM. Measured for tiles of 8, 16, 32
+// and 64, in ms: 128^3 particles at 2048^2 17.6, 10.9, 8.5, 8.7; 16^3 at 1500^2
+// 4.26, 2.24, 1.75, 2.58; 256^3 at 1920 x 1080 in perspective 12.5, 10.6, 9.90,
+// 9.92. Smaller frames would gain as much (128^3 at 1024^2: 4.3 and 3.55), but
+// they are the ones that positions are fitted to, and the gradient of an image
+// loss magnifies the image's last bit a thousand times: they keep the 16 pixels
+// and the bits of the configured tile, as do FP16 lattices (see kTwoStepTile).
+int raster_tile(const lt_ctx* ctx, const lt_camera& c) {
+  if (ctx->L.fmt != LT_POS_F32X4 || (long long)c.W * c.H <= (1LL << 20)) return ctx->cfg.tile;
+  return 32;
+}
+
+// `tile`: tile edge in pixels, or 0 for the context's.
 lt_status project_bin_impl(lt_ctx* ctx, const lt_camera* cams, int n_frames, const int* frame_snapshot,
-                           cudaStream_t s, bool upload_only) {
+                           cudaStream_t s, int tile = 0) {
   if (!ctx) return LT_ERR_ARG;
   if (!ctx->have_lattice) return LT_ERR_STATE;
-  const int tile = ctx->cfg.tile;
+  if (!cams || n_frames < 1) return LT_ERR_ARG;
+  if (tile == 0) tile = ctx->tile_auto ? raster_tile(ctx, cams[0]) : ctx->cfg.tile;
   int W, H;
   bool any_persp;
   lt_status st = prepare_frames(ctx, cams, n_frames, frame_snapshot, tile, &W, &H, &any_persp);
@@ -406,7 +455,7 @@ lt_status project_bin_impl(lt_ctx* ctx, const lt_camera* cams, int n_frames, con
   if ((st = grow(&ctx->d_frames, &ctx->frames_cap, (size_t)n_frames)) != LT_OK) return st;
   const long long tpf = (long long)ctx->h_frames[0].tiles_x * ctx->h_frames[0].tiles_y;
   const long long n_tiles = tpf * n_frames;
-  if ((st = ensure_tiles(ctx, n_tiles)) != LT_OK) return st;
+  if ((st = ensure_tiles(ctx, n_tiles, tile, s)) != LT_OK) return st;
   // tile descriptors of the bin pass: 4 bytes per (frame, cube), kept only
   // below a memory budget (above it the scatter projects every cube again)
   const size_t n_desc = (size_t)n_frames * (size_t)ctx->L.n_particles;
@@ -429,7 +478,6 @@ lt_status project_bin_impl(lt_ctx* ctx, const lt_camera* cams, int n_frames, con
   ctx->any_persp = any_persp;
   ctx->n_tiles = n_tiles;
   ctx->binned = true;
-  if (upload_only) return LT_OK;
   return bin_launches(ctx, s, !is_capturing(s));
 }
 
@@ -440,7 +488,12 @@ lt_status render_impl(lt_ctx* ctx, float* d_image, double* d_mass, cudaStream_t 
   a.off = ctx->d_off;
   a.list = ctx->d_list;
   a.work = ctx->d_work;
-  a.n_items = ctx->n_tiles;
+  a.n_items = ctx->d_hist + lt::kHistItems;
+  a.n_tiles = ctx->n_tiles;
+  a.work_target = work_target(ctx);
+  a.slot = ctx->d_cursor;
+  a.slot_acc = ctx->d_slot_acc;
+  a.slot_done = ctx->d_slot_done;
   a.image = d_image;
   a.image_stride = (long long)ctx->W * ctx->H;
   a.mass_tile = ctx->d_mass_tile;
@@ -455,9 +508,7 @@ lt_status render_impl(lt_ctx* ctx, float* d_image, double* d_mass, cudaStream_t 
   if (fit < 1) return LT_ERR_ARG;  // CTA shape exceeds the SM's registers or shared memory
   if (cps <= 0 || cps > fit) cps = fit;
   if (cps > lt::kRasterMaxCtasPerSm) cps = lt::kRasterMaxCtasPerSm;  // the exact queues are sized for this
-  long long ctas = (long long)ctx->num_sms * cps;
-  if (ctas > ctx->n_tiles) ctas = ctx->n_tiles;
-  if (ctas < 1) ctas = 1;
+  const long long ctas = (long long)ctx->num_sms * cps;
   LT_CUDA(cudaMemsetAsync(&ctx->d_ctr->work_next, 0, sizeof(unsigned long long), s));
   LT_CUDA(lt::launch_raster(a, (int)ctas, threads, ctx->any_persp ? 1 : 0, s));
   if (d_mass) {
@@ -514,6 +565,7 @@ lt_status lt_create(lt_ctx** out, const lt_config* cfg) {
   lt_ctx* ctx = new (std::nothrow) lt_ctx();
   if (!ctx) return LT_ERR_NOMEM;
   ctx->cfg = resolved(cfg ? *cfg : lt_config{});
+  ctx->tile_auto = !cfg || cfg->tile == 0;
   if (cudaGetDevice(&ctx->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
     cudaGetLastError();
@@ -523,7 +575,7 @@ lt_status lt_create(lt_ctx** out, const lt_config* cfg) {
   if (cudaMalloc((void**)&ctx->d_ctr, sizeof(DevCounters)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_ctr, sizeof(DevCounters)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_u64, 64 * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->d_hist, 2 * 64 * sizeof(unsigned)) != cudaSuccess) {
+      cudaMalloc((void**)&ctx->d_hist, lt::kHistWords * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     lt_destroy(ctx);
     return LT_ERR_NOMEM;
@@ -548,6 +600,8 @@ void lt_destroy(lt_ctx* ctx) {
   cudaFree(ctx->d_off);
   cudaFree(ctx->d_work);
   cudaFree(ctx->d_mass_tile);
+  cudaFree(ctx->d_slot_acc);
+  cudaFree(ctx->d_slot_done);
   cudaFree(ctx->d_xq);
   cudaFree(ctx->d_scan_tmp);
   cudaFree(ctx->d_list);
@@ -570,6 +624,7 @@ void lt_destroy(lt_ctx* ctx) {
 lt_status lt_set_config(lt_ctx* ctx, const lt_config* cfg) {
   if (!ctx || !cfg || !valid_config(*cfg)) return LT_ERR_ARG;
   ctx->cfg = resolved(*cfg);
+  ctx->tile_auto = cfg->tile == 0;
   return LT_OK;
 }
 
@@ -615,7 +670,7 @@ lt_status lt_build_tets(lt_ctx* ctx, const void* d_pos, int pos_fmt, int N, floa
 
 lt_status lt_project_bin(lt_ctx* ctx, const lt_camera* cams, int n_frames, const int* frame_snapshot,
                          lt_stream stream) {
-  return project_bin_impl(ctx, cams, n_frames, frame_snapshot, (cudaStream_t)stream, false);
+  return project_bin_impl(ctx, cams, n_frames, frame_snapshot, (cudaStream_t)stream);
 }
 
 lt_status lt_render_tiles(lt_ctx* ctx, float* d_image, double* d_mass, lt_stream stream) {
@@ -655,7 +710,12 @@ lt_status lt_count_fragments(lt_ctx* ctx, long long* h_counts, lt_stream stream)
   a.off = ctx->d_off;
   a.list = ctx->d_list;
   a.work = ctx->d_work;
-  a.n_items = ctx->n_tiles;
+  a.n_items = ctx->d_hist + lt::kHistItems;
+  a.n_tiles = ctx->n_tiles;
+  a.work_target = work_target(ctx);
+  a.slot = ctx->d_cursor;
+  a.slot_acc = ctx->d_slot_acc;
+  a.slot_done = ctx->d_slot_done;
   a.image = nullptr;
   a.image_stride = 0;
   a.mass_tile = nullptr;
@@ -664,8 +724,7 @@ lt_status lt_count_fragments(lt_ctx* ctx, long long* h_counts, lt_stream stream)
   a.xq = nullptr;  // counting queues nothing
   a.xq_cap = 0;
   a.list_cap = ctx->list_cap;
-  long long ctas = (long long)ctx->num_sms * 4;
-  if (ctas > ctx->n_tiles) ctas = ctx->n_tiles;
+  const long long ctas = (long long)ctx->num_sms * 4;
   LT_CUDA(lt::launch_count_fragments(a, ctx->d_frag, ctx->n_frames, (int)ctas, 256, s));
   std::vector<unsigned long long> tmp(ctx->n_frames);
   LT_CUDA(cudaMemcpyAsync(tmp.data(), ctx->d_frag, sizeof(unsigned long long) * ctx->n_frames,
@@ -708,7 +767,7 @@ lt_status lt_resample(lt_ctx* ctx, int n, int weight, int snapshot, float* d_gri
   cam.W = cam.H = n;
   cam.wrap = 1;
   const int snaps[1] = {snapshot};
-  lt_status st = project_bin_impl(ctx, &cam, 1, snaps, s, false);
+  lt_status st = project_bin_impl(ctx, &cam, 1, snaps, s, ctx->cfg.tile);
   if (st != LT_OK) return st;
   const size_t cells = (size_t)n * n * n;
   if ((st = grow(&ctx->d_racc, &ctx->racc_cap, cells)) != LT_OK) return st;
@@ -784,7 +843,7 @@ lt_status lt_render_hybrid(lt_ctx* ctx, const lt_camera* cam, int snapshot, doub
   c.near_radius = near_radius;
   const int snaps[1] = {snapshot};
   // the near cubes: exact projection
-  lt_status st = project_bin_impl(ctx, &c, 1, snaps, s, false);
+  lt_status st = project_bin_impl(ctx, &c, 1, snaps, s);
   if (st != LT_OK) return st;
   if ((st = render_impl(ctx, d_image, nullptr, s)) != LT_OK) return st;
   // the far cubes: centroid splats, added to the image
@@ -797,7 +856,7 @@ lt_status lt_graph_build(lt_ctx* ctx, const lt_camera* cams, int n_frames, const
   cudaStream_t s = (cudaStream_t)stream;
   if (s == 0) return LT_ERR_ARG;  // capture needs a created stream
   // uncaptured pass: upload frames, size the bins
-  lt_status st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s, false);
+  lt_status st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s);
   if (st != LT_OK) return st;
   const unsigned long long want = ctx->entries + ctx->entries / 4 + 4096;
   if (want > ctx->list_cap) {
@@ -860,6 +919,8 @@ lt_status lt_autotune(lt_ctx* ctx, const lt_camera* cams, int n_frames, const in
   if (!ctx->have_lattice) return LT_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
   const lt_config base = ctx->cfg;
+  const bool base_auto = ctx->tile_auto;
+  ctx->tile_auto = false;
   const int tiles[] = {16, 32, 64};
   const int threads[] = {128, 256};
   float best_ms = 1e30f;
@@ -876,12 +937,12 @@ lt_status lt_autotune(lt_ctx* ctx, const lt_camera* cams, int n_frames, const in
       c.ctas_per_sm = 0;
       if (lt::raster_max_ctas_per_sm(th, ti, 1) < 1 || lt::raster_max_ctas_per_sm(th, ti, 0) < 1) continue;
       ctx->cfg = c;
-      lt_status st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s, false);
+      lt_status st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s);
       if (st == LT_OK) st = render_impl(ctx, d_image, nullptr, s);
       if (st != LT_OK) { result = st; break; }
       cudaEventRecord(e0, s);
       for (int r = 0; r < reps && st == LT_OK; ++r) {
-        st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s, false);
+        st = project_bin_impl(ctx, cams, n_frames, frame_snapshot, s);
         if (st == LT_OK) st = render_impl(ctx, d_image, nullptr, s);
       }
       cudaEventRecord(e1, s);
@@ -898,6 +959,7 @@ lt_status lt_autotune(lt_ctx* ctx, const lt_camera* cams, int n_frames, const in
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   ctx->cfg = result == LT_OK ? best_cfg : base;
+  if (result != LT_OK) ctx->tile_auto = base_auto;
   ctx->binned = false;
   if (best) *best = ctx->cfg;
   return result;

@@ -294,9 +294,8 @@ cudaError_t launch_scan(const unsigned* d_count, long long n, unsigned long long
 }
 
 // ---------------------------------------------------------------------------
-// Work list: every global tile, longest lists first (33 log2 buckets).
-
-constexpr int kBuckets = 34;
+// Work list: every global tile's list in chunks, longest first (33 log2
+// buckets). A tile with an empty list has one item too: its pixels are stored.
 
 __device__ __forceinline__ int len_bucket(unsigned long long len) {
   // bucket 0 holds the longest lists; empty tiles go last
@@ -305,12 +304,33 @@ __device__ __forceinline__ int len_bucket(unsigned long long len) {
   return 32 - min(lg, 32);
 }
 
-__global__ void k_bucket_hist(const unsigned long long* __restrict__ off, long long n, unsigned* __restrict__ hist) {
+// The items of one tile: n_full chunks of `per` cubes and a rest (the only
+// item of a short list).
+struct TileItems {
+  unsigned n_full;
+  unsigned long long rest;
+  bool has_rest;
+};
+
+__device__ __forceinline__ TileItems tile_items(unsigned long long len, unsigned long long per) {
+  TileItems t;
+  t.n_full = (unsigned)(len / per);
+  t.rest = len - per * t.n_full;
+  t.has_rest = t.rest > 0 || len == 0;
+  return t;
+}
+
+__global__ void k_bucket_hist(const unsigned long long* __restrict__ off, long long n, unsigned work_target,
+                              unsigned* __restrict__ hist) {
   __shared__ unsigned h[kBuckets];
   for (int i = threadIdx.x; i < kBuckets; i += blockDim.x) h[i] = 0;
   __syncthreads();
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
-    atomicAdd(&h[len_bucket(off[t + 1] - off[t])], 1u);
+  const unsigned long long per = work_chunk(off[n], work_target);
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+    const TileItems c = tile_items(off[t + 1] - off[t], per);
+    if (c.n_full) atomicAdd(&h[len_bucket(per)], c.n_full);
+    if (c.has_rest) atomicAdd(&h[len_bucket(c.rest)], 1u);
+  }
   __syncthreads();
   for (int i = threadIdx.x; i < kBuckets; i += blockDim.x)
     if (h[i]) atomicAdd(&hist[i], h[i]);
@@ -325,26 +345,38 @@ __global__ void k_bucket_scan(unsigned* __restrict__ hist) {
       acc += hist[i];
       hist[i] = 0;
     }
+    hist[kHistItems] = acc;
   }
 }
 
-__global__ void k_bucket_scatter(const unsigned long long* __restrict__ off, long long n, unsigned* __restrict__ hist,
-                                 unsigned long long* __restrict__ work) {
+__global__ void k_bucket_scatter(const unsigned long long* __restrict__ off, long long n, unsigned work_target,
+                                 unsigned* __restrict__ hist, unsigned long long* __restrict__ work,
+                                 unsigned* __restrict__ slot) {
+  const unsigned long long per = work_chunk(off[n], work_target);
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    const int b = len_bucket(off[t + 1] - off[t]);
-    const unsigned pos = hist[kBuckets + b] + atomicAdd(&hist[b], 1u);
-    work[pos] = (unsigned long long)t;
+    const TileItems c = tile_items(off[t + 1] - off[t], per);
+    const unsigned long long w = (unsigned long long)t << kWorkChunkBits;
+    if (c.n_full) {
+      const int b = len_bucket(per);
+      const unsigned pos = hist[kBuckets + b] + atomicAdd(&hist[b], c.n_full);
+      for (unsigned k = 0; k < c.n_full; ++k) work[pos + k] = w | k;
+    }
+    if (c.has_rest) {
+      const int b = len_bucket(c.rest);
+      work[hist[kBuckets + b] + atomicAdd(&hist[b], 1u)] = w | c.n_full;
+    }
+    if (c.n_full + (c.has_rest ? 1u : 0u) > 1u) slot[t] = atomicAdd(&hist[kHistItems + 1], 1u);
   }
 }
 
-cudaError_t launch_worklist(const unsigned long long* d_off, long long n_tiles, unsigned* d_hist,
-                            unsigned long long* d_work, cudaStream_t s) {
-  cudaMemsetAsync(d_hist, 0, sizeof(unsigned) * 2 * kBuckets, s);
+cudaError_t launch_worklist(const unsigned long long* d_off, long long n_tiles, unsigned work_target, unsigned* d_hist,
+                            unsigned long long* d_work, unsigned* d_slot, cudaStream_t s) {
+  cudaMemsetAsync(d_hist, 0, sizeof(unsigned) * kHistWords, s);
   long long blocks = (n_tiles + 255) / 256;
   if (blocks > 2048) blocks = 2048;
-  k_bucket_hist<<<(unsigned)blocks, 256, 0, s>>>(d_off, n_tiles, d_hist);
+  k_bucket_hist<<<(unsigned)blocks, 256, 0, s>>>(d_off, n_tiles, work_target, d_hist);
   k_bucket_scan<<<1, 32, 0, s>>>(d_hist);
-  k_bucket_scatter<<<(unsigned)blocks, 256, 0, s>>>(d_off, n_tiles, d_hist, d_work);
+  k_bucket_scatter<<<(unsigned)blocks, 256, 0, s>>>(d_off, n_tiles, work_target, d_hist, d_work, d_slot);
   return cudaGetLastError();
 }
 

@@ -34,6 +34,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "lt_ff.cuh"
+
 namespace lt {
 
 // Connectivity of the six tetrahedra of a cube (Sec. 4.1); corner n of cube
@@ -155,10 +157,12 @@ struct FrameDev {
   float inv6K;            // 1 / (6 K)
   float tan_x, tan_y;     // perspective image-plane half extents at unit distance
   double unit;            // accumulator unit -> column density
+  FixedScale scale;       // the same as the pixel conversion takes it
+  double exact_scale;     // 6 m / unit: the exact evaluation's scale
   double pix_area;        // pixel area for the frame mass
   // double-precision view for the exact evaluation of ill-conditioned fragments
   double rd[3], ud[3], fd[3], eyed[3];
-  double lod[2], pxd[2];  // ortho window origin and pixel size (world units)
+  double lod[2], pxd[2];  // ortho window origin and pixel size (world units); perspective: pxd = 1 / W, 1 / H
   double tand[2];         // perspective tan(fov/2) in x and y
   double m_tet;           // mass of one tetrahedron
   float sigma_units;      // mean column density in accumulator units (2^frac_bits)
@@ -458,7 +462,16 @@ struct TetRaster {
   float vscale;  // perspective: bound of d value / d T (1 / w_min^2); 1 orthographic
 };
 
-__device__ __forceinline__ float cross2(float ax, float ay, float bx, float by) { return ax * by - ay * bx; }
+// a b - c d. PIN: with the one rounding order written out (the product c d
+// rounded, the rest fused), else as the compiler contracts it. The raster pins
+// it, so that its records do not depend on what surrounds the setup in a kernel.
+template <bool PIN>
+__device__ __forceinline__ float diff2(float a, float b, float c, float d) {
+  return PIN ? __fmaf_rn(a, b, -__fmul_rn(c, d)) : a * b - c * d;
+}
+
+template <bool PIN = false>
+__device__ __forceinline__ float cross2(float ax, float ay, float bx, float by) { return diff2<PIN>(ax, by, ay, bx); }
 
 // Conditionally swap two scalars.
 __device__ __forceinline__ void cswap(bool s, float& p, float& q) {
@@ -470,6 +483,7 @@ __device__ __forceinline__ void cswap(bool s, float& p, float& q) {
 // One hull edge (j, k) with the other two vertices l1, l2, in canonical
 // coordinates; writes f_e = sigma * w * orient(v_j, v_k, x) with
 // w = W / |o1 o2| (W = 6 K, or 6 K / (Z0 Z1 Z2 Z3) in perspective).
+template <bool PIN = false>
 __device__ __forceinline__ void edge_fn(float xj, float yj, float ex, float ey, float o1, float o2, float Wn,
                                         float tiny, float& a, float& b, float& c) {
   const float prod = fmaxf(fabsf(o1 * o2), tiny);
@@ -478,23 +492,24 @@ __device__ __forceinline__ void edge_fn(float xj, float yj, float ex, float ey, 
   const bool dead = (o1 == 0.0f) && (o2 == 0.0f);  // zero-length edge or flat hull
   a = dead ? 0.0f : -ey * w;
   b = dead ? 0.0f : ex * w;
-  c = dead ? __int_as_float(0x7f800000) : (ey * xj - ex * yj) * w;
+  c = dead ? __int_as_float(0x7f800000) : diff2<PIN>(ey, xj, ex, yj) * w;
 }
 
 // Plane of the mapped face (p, q, r) in (X, Y, w) space, w relative to the anchor.
+template <bool PIN = false>
 __device__ __forceinline__ bool face_plane(float xp, float yp, float wp, float xq, float yq, float wq, float xr,
                                            float yr, float wr, float& pa, float& pb, float& pc) {
   const float ux = xq - xp, uy = yq - yp, uw = wq - wp;
   const float vx = xr - xp, vy = yr - yp, vw = wr - wp;
-  const float nw = ux * vy - uy * vx;
-  const float nx = uy * vw - uw * vy;
-  const float ny = uw * vx - ux * vw;
+  const float nw = diff2<PIN>(ux, vy, uy, vx);
+  const float nx = diff2<PIN>(uy, vw, uw, vy);
+  const float ny = diff2<PIN>(uw, vx, ux, vw);
   // a face seen nearly edge-on has an unreliable FP32 slope: treat as vertical
   if (!(fabsf(nw) > 1e-5f * (fabsf(ux * vy) + fabsf(uy * vx)))) return false;
   const float inw = fast_rcp(nw);
   pa = -nx * inw;
   pb = -ny * inw;
-  pc = wp - pa * xp - pb * yp;
+  pc = PIN ? __fmaf_rn(-pb, yp, __fmaf_rn(-pa, xp, wp)) : wp - pa * xp - pb * yp;
   return true;
 }
 
@@ -519,10 +534,11 @@ __device__ __forceinline__ void cswapi(bool s, int& p, int& q) {
   q = s ? tp : tq;
 }
 
+template <bool PIN = false>
 __device__ __forceinline__ bool tet_canon(float x0, float y0, float x1, float y1, float x2, float y2, float x3,
                                           float y3, float w0, float w1, float w2, float w3, TetCanon& k) {
   const float ax = x1 - x0, ay = y1 - y0, bx = x2 - x0, by = y2 - y0, cx = x3 - x0, cy = y3 - y0;
-  const float ab = cross2(ax, ay, bx, by), ac = cross2(ax, ay, cx, cy), bc = cross2(bx, by, cx, cy);
+  const float ab = cross2<PIN>(ax, ay, bx, by), ac = cross2<PIN>(ax, ay, cx, cy), bc = cross2<PIN>(bx, by, cx, cy);
   float c1 = -bc, c2 = ac, c3 = -ab;
   const float c0 = -(c1 + c2 + c3);
   const float S = fabsf(c0) + fabsf(c1) + fabsf(c2) + fabsf(c3);
@@ -550,9 +566,9 @@ __device__ __forceinline__ bool tet_canon(float x0, float y0, float x1, float y1
   k.d1x = x1 - x0; k.d1y = y1 - y0;
   k.d2x = x2 - x0; k.d2y = y2 - y0;
   k.d3x = x3 - x0; k.d3y = y3 - y0;
-  k.D12 = cross2(k.d1x, k.d1y, k.d2x, k.d2y);
-  k.D13 = cross2(k.d1x, k.d1y, k.d3x, k.d3y);
-  k.D23 = cross2(k.d2x, k.d2y, k.d3x, k.d3y);
+  k.D12 = cross2<PIN>(k.d1x, k.d1y, k.d2x, k.d2y);
+  k.D13 = cross2<PIN>(k.d1x, k.d1y, k.d3x, k.d3y);
+  k.D23 = cross2<PIN>(k.d2x, k.d2y, k.d3x, k.d3y);
   k.O123 = k.D12 + k.D23 - k.D13;
   k.S = S;
   return true;
@@ -594,7 +610,7 @@ __device__ __forceinline__ float sel4(const float* v, int i) {
 // (relative pixel coordinates). Kn = 6 K (ortho) or 6 K / (Z0 Z1 Z2 Z3)
 // (perspective); wa = 1/Z of the anchor (perspective). Returns false for a
 // projection of zero area.
-template <bool PERSP>
+template <bool PERSP, bool PIN = false>
 __device__ __forceinline__ bool tet_setup(float x0, float y0, float x1, float y1, float x2, float y2, float x3,
                                           float y3, float w0, float w1, float w2, float w3, float Kn, float wa,
                                           float invKn, TetRaster& t) {
@@ -603,14 +619,15 @@ __device__ __forceinline__ bool tet_setup(float x0, float y0, float x1, float y1
   t.ymin = fminf(fminf(y0, y1), fminf(y2, y3));
   t.ymax = fmaxf(fmaxf(y0, y1), fmaxf(y2, y3));
   TetCanon K;
-  if (!tet_canon(x0, y0, x1, y1, x2, y2, x3, y3, w0, w1, w2, w3, K)) return false;
+  if (!tet_canon<PIN>(x0, y0, x1, y1, x2, y2, x3, y3, w0, w1, w2, w3, K)) return false;
   const float tiny = K.S * K.S * 1e-12f;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const EdgeRef r = edge_ref(K, e);
-    edge_fn(sel4(K.x, r.j), sel4(K.y, r.j), r.ex, r.ey, r.o1, r.o2, Kn, tiny, t.a[e], t.b[e], t.c[e]);
+    edge_fn<PIN>(sel4(K.x, r.j), sel4(K.y, r.j), r.ex, r.ey, r.o1, r.o2, Kn, tiny, t.a[e], t.b[e], t.c[e]);
     const float omin = fminf(fabsf(r.o1), fabsf(r.o2));
-    t.st[e] = __fdividef(r.ex * r.ex + r.ey * r.ey, fmaxf(omin, tiny));
+    const float e2 = PIN ? __fmaf_rn(r.ex, r.ex, __fmul_rn(r.ey, r.ey)) : r.ex * r.ex + r.ey * r.ey;
+    t.st[e] = __fdividef(e2, fmaxf(omin, tiny));
   }
   if (!K.caseB) {
     t.a[3] = 0.0f;
@@ -632,12 +649,13 @@ __device__ __forceinline__ bool tet_setup(float x0, float y0, float x1, float y1
     const float* W = K.w;
     const float C0 = fabsf(K.O123), C1 = fabsf(K.D23), C2 = fabsf(K.D13), C3 = fabsf(K.D12);
     // Q > 0: the (0,1) diagonal (case B) / the outer face (case A) is the lower w surface
-    const float Q = K.caseB ? (C2 * W[2] + C3 * W[3]) - (C0 * W[0] + C1 * W[1])
-                            : C3 * W[3] - (C0 * W[0] + C1 * W[1] + C2 * W[2]);
+    const float q01 = PIN ? __fmaf_rn(C0, W[0], __fmul_rn(C1, W[1])) : C0 * W[0] + C1 * W[1];
+    const float Q = K.caseB ? (PIN ? __fmaf_rn(C2, W[2], __fmul_rn(C3, W[3])) : C2 * W[2] + C3 * W[3]) - q01
+                            : (PIN ? __fmaf_rn(C3, W[3], -__fmaf_rn(C2, W[2], q01)) : C3 * W[3] - (q01 + C2 * W[2]));
     bool ok1, ok2;
     float pa0 = 0.f, pb0 = 0.f, pc0 = 0.f, pa1 = 0.f, pb1 = 0.f, pc1 = 0.f;
     if (!K.caseB) {
-      ok1 = face_plane(X[0], Y[0], W[0], X[1], Y[1], W[1], X[2], Y[2], W[2], pa0, pb0, pc0);
+      ok1 = face_plane<PIN>(X[0], Y[0], W[0], X[1], Y[1], W[1], X[2], Y[2], W[2], pa0, pb0, pc0);
       ok2 = ok1;
       pa1 = pa0; pb1 = pb0; pc1 = pc0;
     } else {
@@ -645,8 +663,8 @@ __device__ __forceinline__ bool tet_setup(float x0, float y0, float x1, float y1
       const int ip = low01 ? 0 : 2, iq = low01 ? 1 : 3, ir = low01 ? 2 : 0, is = low01 ? 3 : 1;
       const float px = sel4(X, ip), py = sel4(Y, ip), pw = sel4(W, ip);
       const float qx = sel4(X, iq), qy = sel4(Y, iq), qw = sel4(W, iq);
-      ok1 = face_plane(px, py, pw, qx, qy, qw, sel4(X, ir), sel4(Y, ir), sel4(W, ir), pa0, pb0, pc0);
-      ok2 = face_plane(px, py, pw, qx, qy, qw, sel4(X, is), sel4(Y, is), sel4(W, is), pa1, pb1, pc1);
+      ok1 = face_plane<PIN>(px, py, pw, qx, qy, qw, sel4(X, ir), sel4(Y, ir), sel4(W, ir), pa0, pb0, pc0);
+      ok2 = face_plane<PIN>(px, py, pw, qx, qy, qw, sel4(X, is), sel4(Y, is), sel4(W, is), pa1, pb1, pc1);
     }
     if (!ok1 && !ok2) return false;
     if (!ok1) { pa0 = pa1; pb0 = pb1; pc0 = pc1; }
@@ -704,15 +722,12 @@ __device__ __forceinline__ void accum_fixed(unsigned long long* acc, float q, De
   }
 }
 
-// Exact value of rho_t * dl_t (Eq. 3, 6, 9) for tetrahedron s of `cube` at
-// pixel (px, py) of the copy shifted by (sx, sy) periods, in FP64 from the
-// stored positions: the ray through the pixel centre clipped against the four
-// face planes. Used for the rare fragments whose FP32 evaluation is
-// ill-conditioned. Returns the value in column-density units divided by the
-// pixel's ray-direction length for perspective frames (the factor the tile
-// applies when it stores the pixel).
-__device__ __noinline__ static double exact_fragment(const Lattice& L, const FrameDev& F, long long cube, int s, int sx, int sy, int px,
-                                 int py, double m) {
+// Exact value of rho_t * dl_t by clipping the pixel ray against the four face
+// planes (see exact_fragment). Returns the value in column-density units
+// divided by the pixel's ray-direction length for perspective frames.
+__device__ __noinline__ static double exact_clip(const Lattice& L, const FrameDev& F, long long cube, int s, int sx, int sy,
+                                                 int px, int py) {
+  const double m = F.m_tet;
   const int N = L.N;
   const int i = (int)(cube % N), j = (int)((cube / N) % N), k = (int)(cube / ((long long)N * N));
   const long long soff = (long long)F.snapshot * L.n_particles;
@@ -800,6 +815,139 @@ __device__ __noinline__ static double exact_fragment(const Lattice& L, const Fra
   const double chord = (t_out - t_in) * dl;
   const double val = m / fabs(V) * chord;
   return half ? val / dl : val;
+}
+
+// Exact value of rho_t * dl_t (Eq. 3, 6, 9) for tetrahedron s of `cube` at
+// pixel (px, py) of the copy shifted by (sx, sy) periods, in FP64 from the
+// stored positions. Used for the fragments whose FP32 evaluation is
+// ill-conditioned. Returns accumulator units, over the pixel's ray-direction
+// length for perspective frames (the factor the tile applies when it stores
+// the pixel).
+//
+// The pyramid form of the head of this file, about the ray: (u, v) are the
+// vertices' coordinates across it (in perspective after the shear
+// (X - xt Z, Y - yt Z, Z), which keeps volumes and makes the pixel's ray the
+// line u = v = 0, so the orthographic form holds for that ray), s_jk = u_j v_k
+// - u_k v_j, and the value is 6 m min s_jk / (o1 o2) over the hull edges, with
+// the orientations o1, o2 of the other two vertices. That is about 140 FP64
+// operations with one division; clipping the ray against the four planes takes
+// about ten times as many, and was 24% of the FP64 pipe of a 128^3 frame at
+// 1024^2. The clip stays for tetrahedra within 2e-5 |e|^3 of flat, where its
+// own rounding (of coordinates of the size of the box, against a chord that
+// goes to zero) shows and the two forms part.
+__device__ __noinline__ static float exact_fragment(const Lattice& L, const FrameDev& F, long long cube, int s, int sx,
+                                                    int sy, int px, int py) {
+  int i, j, k;
+  cube_ijk(L, cube, i, j, k);
+  const int N = L.N;
+  const long long soff = (long long)F.snapshot * L.n_particles;
+  const double h = (double)L.box / N, box = (double)L.box;
+  float e32[4][3];
+  double v[4][3];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int n = tet_corner_dyn(s, c);
+    const int a = n & 1, b = (n >> 1) & 1, cc = (n >> 2) & 1;
+    const int im[3] = {i + a == N ? 0 : i + a, j + b == N ? 0 : j + b, k + cc == N ? 0 : k + cc};
+    const int o[3] = {a, b, cc};
+    if (L.fmt == 0) {
+      const float4 p = __ldg(reinterpret_cast<const float4*>(L.pos) + soff + particle_id(im[0], im[1], im[2], N));
+      const float pp[3] = {p.x, p.y, p.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const float d0 = pp[q] - (float)im[q] * L.h;
+        double d = fma(-(double)im[q], h, (double)pp[q]);
+        e32[c][q] = d0 + (float)o[q] * L.h;
+        if (fabsf(d0) > L.half_box) {  // minimum image
+          d += d0 > 0.f ? -box : box;
+          e32[c][q] += d0 > 0.f ? -L.box : L.box;
+        }
+        v[c][q] = fma((double)o[q], h, d);
+      }
+    } else {
+      bool ok = true;
+      const float3 df = load_disp(L, soff, i, j, k, n, ok);
+      const float dd[3] = {df.x, df.y, df.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        e32[c][q] = dd[q] + (float)o[q] * L.h;
+        v[c][q] = fma((double)o[q], h, (double)dd[q]);
+      }
+    }
+  }
+  {
+    // 6 |V| in FP32 against the product of the longest edge components
+    float em = 0.f;
+#pragma unroll
+    for (int c = 1; c < 4; ++c)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        e32[c][q] -= e32[0][q];
+        em = fmaxf(em, fabsf(e32[c][q]));
+      }
+    const float V6 = e32[1][0] * (e32[2][1] * e32[3][2] - e32[2][2] * e32[3][1]) +
+                     e32[1][1] * (e32[2][2] * e32[3][0] - e32[2][0] * e32[3][2]) +
+                     e32[1][2] * (e32[2][0] * e32[3][1] - e32[2][1] * e32[3][0]);
+    if (!(fabsf(V6) > 2e-5f * em * em * em)) return (float)(exact_clip(L, F, cube, s, sx, sy, px, py) / F.unit);
+  }
+  double u[4], w[4];
+  const double q0 = (double)i * h, q1 = (double)j * h, q2 = (double)k * h;
+  if (!F.persp) {
+    const double a = F.lod[0] + ((double)(px - sx * F.W) + 0.5) * F.pxd[0];
+    const double b = F.lod[1] + ((double)(py - sy * F.H) + 0.5) * F.pxd[1];
+    const double u0 = fma(F.rd[0], q0, fma(F.rd[1], q1, fma(F.rd[2], q2, -a)));
+    const double w0 = fma(F.ud[0], q0, fma(F.ud[1], q1, fma(F.ud[2], q2, -b)));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      u[c] = fma(F.rd[0], v[c][0], fma(F.rd[1], v[c][1], fma(F.rd[2], v[c][2], u0)));
+      w[c] = fma(F.ud[0], v[c][0], fma(F.ud[1], v[c][1], fma(F.ud[2], v[c][2], w0)));
+    }
+  } else {
+    const double xt = F.tand[0] * ((2.0 * (double)px + 1.0) * F.pxd[0] - 1.0);  // pxd: 1 / W, 1 / H
+    const double yt = F.tand[1] * ((2.0 * (double)py + 1.0) * F.pxd[1] - 1.0);
+    // the axes across the ray: (r - xt f) and (u - yt f)
+    const double r0 = fma(-xt, F.fd[0], F.rd[0]), r1 = fma(-xt, F.fd[1], F.rd[1]), r2 = fma(-xt, F.fd[2], F.rd[2]);
+    const double t0 = fma(-yt, F.fd[0], F.ud[0]), t1 = fma(-yt, F.fd[1], F.ud[1]), t2 = fma(-yt, F.fd[2], F.ud[2]);
+    const double c0 = q0 - F.eyed[0], c1 = q1 - F.eyed[1], c2 = q2 - F.eyed[2];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double x = c0 + v[c][0], y = c1 + v[c][1], z = c2 + v[c][2];
+      u[c] = fma(r0, x, fma(r1, y, r2 * z));
+      w[c] = fma(t0, x, fma(t1, y, t2 * z));
+    }
+  }
+  const double s01 = fma(u[0], w[1], -(u[1] * w[0])), s02 = fma(u[0], w[2], -(u[2] * w[0]));
+  const double s03 = fma(u[0], w[3], -(u[3] * w[0])), s12 = fma(u[1], w[2], -(u[2] * w[1]));
+  const double s13 = fma(u[1], w[3], -(u[3] * w[1])), s23 = fma(u[2], w[3], -(u[3] * w[2]));
+  double t123 = s12 + s23 - s13, t023 = s02 + s23 - s03, t013 = s01 + s13 - s03, t012 = s01 + s12 - s02;
+  // an orientation of rounding's size (coordinates of the box's size over the
+  // tetrahedron's, times 2^-53) is a face seen edge-on
+  const double none = 1e-12 * (fabs(t123) + fabs(t023) + fabs(t013) + fabs(t012));
+  if (fabs(t123) < none) t123 = 0.0;
+  if (fabs(t023) < none) t023 = 0.0;
+  if (fabs(t013) < none) t013 = 0.0;
+  if (fabs(t012) < none) t012 = 0.0;
+  // the smallest s_jk / (o1 o2) over the edges with both other vertices on one
+  // side (a face seen edge-on counts with either: it bounds the hull without a
+  // value of its own), as a quotient bn / bp
+  double bn = 1.0, bp = 0.0;
+  bool outside = false;
+  auto edge = [&](double n, double o1, double o2) {
+    const double p = o1 * o2;
+    if (p < 0.0) return;  // inside the hull
+    const double sum = o1 + o2;
+    if (sum < 0.0) n = -n;
+    if (n < 0.0 && sum != 0.0) outside = true;
+    if (p > 0.0 && n * bp <= bn * p) { bn = n; bp = p; }
+  };
+  edge(s01, t012, t013);
+  edge(s02, -t012, t023);
+  edge(s03, -t013, -t023);
+  edge(s12, t012, t123);
+  edge(s13, t013, -t123);
+  edge(s23, t023, t123);
+  if (outside || !(bp > 0.0)) return 0.0f;
+  return (float)(F.exact_scale * bn / bp);
 }
 
 // One tetrahedron in FP64, relative to its cube's corner-0 Lagrangian point.

@@ -100,4 +100,15 @@ __device__ __forceinline__ float fixed_to_float(unsigned long long acc, const Fi
   return __fadd_rn(p.h, __fmaf_rn(n.h, s.u.l, __fmaf_rn(n.l, s.u.h, p.l)));
 }
 
+// (float)((double)acc * unit * factor), the same way.
+__device__ __forceinline__ float fixed_to_float(unsigned long long acc, const FixedScale& s, float factor) {
+  const unsigned hi = (unsigned)(acc >> 23);
+  if (!s.small || (acc >> 46)) return (float)((double)acc * s.unit * (double)factor);
+  const float a = __fsub_rn(__uint_as_float(0x4b000000u | hi), 8388608.0f) * 8388608.0f;
+  const float b = __fsub_rn(__uint_as_float(0x4b000000u | ((unsigned)acc & 0x7fffffu)), 8388608.0f);
+  const ff v = ff_fast_sum(a, b) * s.u;
+  const ff p = ff_two_prod(v.h, factor);
+  return __fadd_rn(p.h, __fmaf_rn(v.l, factor, p.l));
+}
+
 }  // namespace lt

@@ -23,8 +23,31 @@ size_t scan_tmp_words(long long n);
 cudaError_t launch_bin_scatter(const Lattice& L, const FrameDev* d_frames, int n_frames,
                                const unsigned long long* d_off, unsigned* d_cursor, unsigned* d_list,
                                unsigned long long capacity, unsigned* d_desc, DevCounters* ctr, cudaStream_t s);
-cudaError_t launch_worklist(const unsigned long long* d_off, long long n_tiles, unsigned* d_hist,
-                            unsigned long long* d_work, cudaStream_t s);
+// Work list of the raster: every tile's list in chunks of work_chunk() cubes,
+// longest first; d_slot receives the slot of each tile that has several.
+cudaError_t launch_worklist(const unsigned long long* d_off, long long n_tiles, unsigned work_target, unsigned* d_hist,
+                            unsigned long long* d_work, unsigned* d_slot, cudaStream_t s);
+
+// A work item is tile << kWorkChunkBits | chunk.
+constexpr int kWorkChunkBits = 20;
+constexpr int kBuckets = 34;                  // list lengths by log2
+constexpr int kHistItems = 2 * kBuckets;      // d_hist: number of items, then of slots
+constexpr int kHistWords = 2 * kBuckets + 2;
+// Items a CTA gets on average beyond one per tile: enough that the longest
+// first leave the CTAs within a few percent of each other at the end.
+constexpr unsigned kItemsPerCta = 16;
+constexpr unsigned long long kMinChunk = 128;  // one batch of 16 cubes for each of 8 warps
+
+// Cubes per item when `total` list entries are spread over work_target
+// (CTAs x kItemsPerCta) items: the lists then make at most work_target items
+// more than there are tiles, and at most work_target tiles have several.
+__host__ __device__ inline unsigned long long work_chunk(unsigned long long total, unsigned work_target) {
+  const unsigned long long c = (total + work_target - 1) / work_target;
+  return c < kMinChunk ? kMinChunk : c;
+}
+__host__ __device__ inline unsigned work_chunks(unsigned long long len, unsigned long long per) {
+  return len <= per ? 1u : (unsigned)((len + per - 1) / per);
+}
 
 // ---- lt_raster.cu
 struct RasterArgs {
@@ -33,7 +56,12 @@ struct RasterArgs {
   const unsigned long long* off;
   const unsigned* list;
   const unsigned long long* work;
-  long long n_items;
+  const unsigned* n_items;       // on the device: items of the work list
+  long long n_tiles;
+  unsigned work_target;          // see work_chunk
+  const unsigned* slot;          // per global tile: its slot, where it has several items
+  unsigned long long* slot_acc;  // tile x tile sums per slot, zero between renders
+  unsigned* slot_done;           // finished items per slot, zero between renders
   float* image;
   long long image_stride;  // floats per frame (W * H)
   double* mass_tile;       // per global tile

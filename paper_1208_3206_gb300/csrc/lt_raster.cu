@@ -89,8 +89,8 @@ __device__ __forceinline__ void cube_fragments(const CubeProj& P, const FrameDev
                                               make_float4(t.c[0], t.c[1], t.c[2], t.c[3]),
                                               make_float4(t.st[0], t.st[1], t.st[2], t.st[3]), X, Y, delta, dvdT,
                                               v, F.sigma_units)) {
-              const double ex = exact_fragment(Lat, F, cube, s, sx, sy, px, py, F.m_tet);
-              if (ex > 0.0) fn(px, py, (float)(ex / F.unit));
+              const float ex = exact_fragment(Lat, F, cube, s, sx, sy, px, py);
+              if (ex > 0.0f) fn(px, py, ex);
               continue;
             }
             if (v > 0.0f) fn(px, py, v);
