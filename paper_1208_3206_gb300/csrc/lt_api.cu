@@ -532,8 +532,7 @@ lt_status centroids_impl(lt_ctx* ctx, const lt_camera& cam, int snapshot, float*
   ctx->h_frames[0] = F;
   LT_CUDA(cudaMemcpyAsync(ctx->d_frame_cen, ctx->h_frames, sizeof(FrameDev), cudaMemcpyHostToDevice, s));
   // the fixed-point unit is the frame's: 2^-frac_bits of its mean column density
-  LT_CUDA(lt::launch_centroids(ctx->L, ctx->d_frame_cen, cam.W, cam.H, F.m_tet, F.unit, ctx->d_cacc, d_image, add,
-                               ctx->d_ctr, s));
+  LT_CUDA(lt::launch_centroids(ctx->L, F, ctx->d_frame_cen, ctx->d_cacc, d_image, add, ctx->d_ctr, s));
   LT_CUDA(cudaStreamSynchronize(s));
   return LT_OK;
 }

@@ -411,7 +411,7 @@ cudaError_t launch_area(const Lattice& L, const FrameDev* d_frame, int W, int H,
   k_area<<<(unsigned)(blocks < 1 ? 1 : blocks), kAreaThreads, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_fixed_finalize(d_acc, np, unit, false, d_out, s);
+  return launch_fixed_finalize(d_acc, np, unit, false, nullptr, d_out, s);
 }
 
 }  // namespace lt

@@ -1009,6 +1009,67 @@ __device__ __forceinline__ void tet_f64(const Lattice& L, long long soff, int i,
   }
 }
 
+// One tetrahedron in float-float, relative to its cube's Lagrangian corner
+// (i h, j h, k h): a vertex is the stored position minus that corner, unwrapped
+// (h_ff = box / N as a pair; a corner past the last lattice plane is one
+// period further, which makes it the position plus h).
+__device__ __forceinline__ void tet_ff(const Lattice& L, ff h_ff, long long soff, int i, int j, int k, int s, bool& ok,
+                                       ff (&v)[4][3]) {
+  const int N = L.N, idx[3] = {i, j, k};
+  ff q0[3];
+  float qf[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float f = (float)idx[q];
+    const ff p = ff_two_prod(f, h_ff.h);
+    q0[q] = ff_fast_sum(p.h, __fmaf_rn(f, h_ff.l, p.l));
+    qf[q] = f * L.h;
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int n = tet_corner_dyn(s, c);
+    const int o[3] = {n & 1, (n >> 1) & 1, n >> 2};
+    if (L.fmt == 0) {
+      const int im = i + o[0] == N ? 0 : i + o[0], jm = j + o[1] == N ? 0 : j + o[1], km = k + o[2] == N ? 0 : k + o[2];
+      const float4 p4 = __ldg(reinterpret_cast<const float4*>(L.pos) + soff + particle_id(im, jm, km, N));
+      const float p[3] = {p4.x, p4.y, p4.z};
+      ok = ok && isfinite(p4.x) && isfinite(p4.y) && isfinite(p4.z);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const bool past = idx[q] + o[q] == N;
+        const ff d = ff_two_sum(p[q], past ? h_ff.h : -q0[q].h);
+        v[c][q] = ff_fast_sum(d.h, __fadd_rn(d.l, past ? h_ff.l : -q0[q].l));
+        const float d0 = p[q] - (past ? 0.f : qf[q] + (float)o[q] * L.h);  // displacement
+        if (fabsf(d0) > L.half_box) v[c][q] = v[c][q] + (d0 > 0.f ? -L.box : L.box);
+      }
+    } else {
+      const float3 df = load_disp(L, soff, i, j, k, n, ok);
+      const float d[3] = {df.x, df.y, df.z};
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const ff e = ff_two_sum(d[q], o[q] ? h_ff.h : 0.f);
+        v[c][q] = ff_fast_sum(e.h, __fadd_rn(e.l, o[q] ? h_ff.l : 0.f));
+      }
+    }
+  }
+}
+
+// Six times the signed volume of a float-float tetrahedron; false when it
+// cancels so far (below 2^-18 of its terms) that FP64 has to take it.
+__device__ __forceinline__ bool volume6_ff(const ff (&v)[4][3], ff& det) {
+  ff e[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) e[c][q] = v[c + 1][q] - v[0][q];
+  det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) + e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
+        e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
+  const float mag = fabsf(e[0][0].h) * (fabsf(e[1][1].h * e[2][2].h) + fabsf(e[1][2].h * e[2][1].h)) +
+                    fabsf(e[0][1].h) * (fabsf(e[1][2].h * e[2][0].h) + fabsf(e[1][0].h * e[2][2].h)) +
+                    fabsf(e[0][2].h) * (fabsf(e[1][0].h * e[2][1].h) + fabsf(e[1][1].h * e[2][0].h));
+  return fabsf(det.h) >= mag * (1.0f / 262144.0f) && fabsf(det.h) > 1e-30f;
+}
+
 // Error model of a fragment's FP32 value (accumulator units). Every hull edge
 // e gets a bound e_e on its FP32 edge function f_e:
 //   * the rounding of the projected vertex positions, absolute: the edge

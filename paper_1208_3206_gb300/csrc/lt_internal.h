@@ -95,15 +95,16 @@ cudaError_t launch_resample(const Lattice& L, const FrameDev* d_frame, long long
 cudaError_t launch_slice(const Lattice& L, int snapshot, int n, int weight, double z0, double m_tet, double unit,
                          unsigned long long* d_acc, float* d_out, DevCounters* ctr, cudaStream_t s);
 
-// ---- lt_centroids.cu: centroid splats of one orthographic frame.
+// ---- lt_centroids.cu: centroid splats of one frame (F, and its copy on the device).
 // `add`: add to d_out instead of overwriting it. With F.near_r2 > 0 only
 // the far cubes (cube_far) are drawn.
-cudaError_t launch_centroids(const Lattice& L, const FrameDev* d_frame, int W, int H, double m_tet, double unit,
-                             unsigned long long* d_acc, float* d_out, bool add, DevCounters* ctr, cudaStream_t s);
+cudaError_t launch_centroids(const Lattice& L, const FrameDev& F, const FrameDev* d_frame, unsigned long long* d_acc,
+                             float* d_out, bool add, DevCounters* ctr, cudaStream_t s);
 // 64-bit fixed-point sums (units of `unit`) to float, overwriting or adding to
 // d_out (the last step of every kernel that sums in global memory).
-cudaError_t launch_fixed_finalize(const unsigned long long* d_acc, long long np, double unit, bool add, float* d_out,
-                                  cudaStream_t s);
+// With d_frame (a perspective view) times each pixel's ray-direction length.
+cudaError_t launch_fixed_finalize(const unsigned long long* d_acc, long long np, double unit, bool add,
+                                  const FrameDev* d_frame, float* d_out, cudaStream_t s);
 
 // ---- lt_area.cu: area-averaged pixels of one orthographic frame.
 cudaError_t launch_area(const Lattice& L, const FrameDev* d_frame, int W, int H, double m_tet, double unit,

@@ -224,7 +224,7 @@ cudaError_t launch_resample(const Lattice& L, const FrameDev* d_frame, long long
   k_resample<<<(unsigned)n_tiles, kResampleThreads, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_fixed_finalize(d_acc, cells, unit, false, d_out, s);
+  return launch_fixed_finalize(d_acc, cells, unit, false, nullptr, d_out, s);
 }
 
 }  // namespace lt

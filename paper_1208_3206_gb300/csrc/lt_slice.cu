@@ -346,7 +346,7 @@ cudaError_t launch_slice(const Lattice& L, int snapshot, int n, int weight, doub
   k_slice<<<(unsigned)(blocks < 1 ? 1 : blocks), kSliceThreads, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_fixed_finalize(d_acc, np, unit, false, d_out, s);
+  return launch_fixed_finalize(d_acc, np, unit, false, nullptr, d_out, s);
 }
 
 }  // namespace lt

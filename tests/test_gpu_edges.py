@@ -62,6 +62,14 @@ def unwrapped(pos, N, box):
     return d - box * np.round(d / box)
 
 
+def decoded(off, N):
+    """The positions that FP16 offsets stand for in a unit box: the offset
+    times the cell edge as the renderer holds it, in FP32."""
+    i = np.arange(N ** 3)
+    q = np.stack([i % N, (i // N) % N, i // (N * N)], axis=1) / N
+    return np.mod(q + (off[:, :3].astype(np.float32) * (np.float32(1) / np.float32(N))).astype(np.float64), 1.0)
+
+
 @pytest.mark.parametrize("N,box,half,snaps", [(1, 1.0, False, 1), (2, 1.0, False, 3), (3, 1.0, False, 2), (7, 100.0, False, 3),
                                               (8, 1.0, True, 1), (16, 1.0, False, 2), (33, 1.0, False, 1),
                                               (33, 40.0, True, 2), (64, 1.0, False, 1)])
@@ -124,9 +132,7 @@ def test_slices(R, N, n, z0, half, weight):
     d = lattice(N, 1.7, 5)
     if half:
         p = fp16_offsets(d, N)
-        i = np.arange(N ** 3)
-        q = np.stack([i % N, (i // N) % N, i // (N * N)], axis=1) / N
-        ref_pos = np.mod(q + p[:, :3].astype(np.float64) / N, 1.0)
+        ref_pos = decoded(p, N)
     else:
         p = ref_pos = wrapped(d, N, 1.0)
     R.build_tets(torch.from_numpy(p).cuda(), N)
@@ -176,3 +182,30 @@ def test_raster_items(kind, N, W, H, tile, frac_bits):
     assert abs(float(mass[0]) - ref.sum() * area) <= 1e-5 * ref.sum() * area
     r.project_bin([cam])  # fewer tiles in the same buffers
     assert torch.equal(r.render_tiles()[0], img[0])
+
+
+@pytest.mark.parametrize("N,W,H,kind,lam,half", [(1, 9, 7, "z", 0.5, False), (3, 40, 33, "z", 1.0, False), (13, 300, 7, "z", 2.0, False),
+                                                 (49, 61, 50, "z", 3.0, False), (50, 64, 48, "persp", 2.0, False),
+                                                 (16, 256, 256, "persp", 4.0, False), (20, 90, 80, "z", 6.0, True)])
+def test_centroid_blocks(N, W, H, kind, lam, half):
+    """Splats by blocks of the lattice: blocks that the lattice does not fill,
+    several windows per block (splats of 100 pixels and more), blocks strewn by
+    strong displacement, both block sizes, periodic copies. A pixel's sum is
+    off by the FP32 spline (a few 2^-24 each) and 2^-28 of the mean: 1e-5."""
+    from paper_1208_3206_gb300.render import Renderer
+    r = Renderer()
+    d = lattice(N, lam, 9)
+    if half:
+        p = fp16_offsets(d, N)
+        ref_pos = decoded(p, N)
+    else:
+        p = ref_pos = wrapped(d, N, 1.0)
+    cam = view(W, H, kind)
+    r.build_tets(torch.from_numpy(p).cuda(), N)
+    img = r.render_centroids(cam)
+    again = r.render_centroids(cam)
+    r.sync()
+    ref = oracle.centroids(ref_pos, N, cam)
+    got = img.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
+    assert torch.equal(img, again)
