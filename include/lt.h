@@ -245,15 +245,12 @@ lt_status lt_render_backward(lt_ctx* ctx, const float* d_dL_dimage, float* d_dL_
  * (every periodic copy of t counts). weight LT_WEIGHT_DENSITY: q_t = rho_t
  * (Eq. 3), so a cell holds rho dl, its mass over its face area;
  * LT_WEIGHT_STREAMS: q_t = 1, so a cell over g is the mean number of streams
- * on its line. Each (tetrahedron, line) interval is found exactly in FP64 by
- * clipping the line against the four face planes; the cells are summed as
+ * on its line. Each (tetrahedron, line) interval is found by clipping the
+ * line against the four face planes, to about 2^-40 of a cell; the cells are summed as
  * 64-bit fixed-point integers (2^-frac_bits of the mean cell), so the grid
  * is bitwise reproducible. Tetrahedra with V == 0 contribute nothing.
- * Uses the project-and-bin pass with an orthographic view along z whose
- * pixels are the grid's columns, so it replaces the frames and bins of the
- * last lt_project_bin (render or count afterwards only after a new
- * lt_project_bin), synchronises once to size the bins, and keeps an n^3
- * array of 64-bit cells in the context.
+ * Asynchronous; leaves the bins of the last lt_project_bin untouched; keeps an
+ * n^3 array of 64-bit cells in the context.
  * Errors: LT_ERR_STATE (no lt_build_tets), LT_ERR_ARG (null d_grid, n < 1 or
  * n > 2048, unknown weight, snapshot out of range), LT_ERR_NOMEM; a cell
  * leaving the fixed-point range latches LT_ERR_RANGE.

@@ -755,19 +755,7 @@ lt_status lt_resample(lt_ctx* ctx, int n, int weight, int snapshot, float* d_gri
   if (!ctx->have_lattice) return LT_ERR_STATE;
   if (snapshot < 0 || snapshot >= ctx->n_snap) return LT_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  // the grid's columns are the pixels of an orthographic view along z over
-  // the periodic box window: pixel (a, b) is centred on column (a, b)
-  lt_camera cam;
-  memset(&cam, 0, sizeof cam);
-  cam.type = LT_ORTHO;
-  cam.fwd[2] = 1.0;
-  cam.up[1] = 1.0;
-  cam.hi[0] = cam.hi[1] = ctx->L.box;
-  cam.W = cam.H = n;
-  cam.wrap = 1;
-  const int snaps[1] = {snapshot};
-  lt_status st = project_bin_impl(ctx, &cam, 1, snaps, s, ctx->cfg.tile);
-  if (st != LT_OK) return st;
+  lt_status st;
   const size_t cells = (size_t)n * n * n;
   if ((st = grow(&ctx->d_racc, &ctx->racc_cap, cells)) != LT_OK) return st;
   const double box = ctx->L.box, gs = box / n;
@@ -778,8 +766,7 @@ lt_status lt_resample(lt_ctx* ctx, int n, int weight, int snapshot, float* d_gri
   const double mean_cell = weight == LT_WEIGHT_DENSITY ? ctx->total_mass / (box * box * box) * gs : gs;
   const double unit = mean_cell / ldexp(1.0, ctx->cfg.frac_bits);
   LT_CUDA(cudaMemsetAsync(&ctx->d_ctr->resample_intervals, 0, 2 * sizeof(unsigned long long), s));
-  LT_CUDA(lt::launch_resample(ctx->L, ctx->d_frames, ctx->n_tiles, ctx->tile, ctx->d_off, ctx->d_list, ctx->list_cap,
-                              n, weight, m_tet, unit, ctx->d_racc, d_grid, ctx->d_ctr, s));
+  LT_CUDA(lt::launch_resample(ctx->L, snapshot, n, weight, m_tet, unit, ctx->d_racc, d_grid, ctx->d_ctr, s));
   return LT_OK;
 }
 

@@ -83,12 +83,9 @@ cudaError_t launch_atomic(const Lattice& L, const FrameDev* d_frames, long long 
                           DevCounters* ctr, cudaStream_t s);
 
 // ---- lt_resample.cu: resampling onto a periodic n^3 grid (q = rho: weight 0,
-// q = 1: weight 1) from the bins of an orthographic view along z whose
-// pixels are the grid's columns.
-cudaError_t launch_resample(const Lattice& L, const FrameDev* d_frame, long long n_tiles, int tile,
-                            const unsigned long long* d_off, const unsigned* d_list, unsigned long long list_cap, int n,
-                            int weight, double m_tet, double unit, unsigned long long* d_acc, float* d_out,
-                            DevCounters* ctr, cudaStream_t s);
+// q = 1: weight 1).
+cudaError_t launch_resample(const Lattice& L, int snapshot, int n, int weight, double m_tet, double unit,
+                            unsigned long long* d_acc, float* d_out, DevCounters* ctr, cudaStream_t s);
 
 // ---- lt_slice.cu: total density (weight 0) or stream count (weight 1) at
 // the centres of an n x n grid on the plane z = z0.

@@ -209,3 +209,32 @@ def test_centroid_blocks(N, W, H, kind, lam, half):
     got = img.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
     assert torch.equal(img, again)
+
+
+@pytest.mark.parametrize("N,n,lam,half", [(1, 4, 0.5, False), (2, 33, 1.0, False), (5, 1, 1.0, False), (6, 70, 2.0, False),
+                                          (11, 24, 3.0, False), (33, 8, 3.0, False), (16, 40, 4.0, True), (12, 31, 0.0, False)])
+@pytest.mark.parametrize("weight", ["density", "streams"])
+def test_resample_forms(N, n, lam, half, weight):
+    """Cells against the oracle: columns past the periodic edge, tetrahedra of
+    hundreds of columns and cells and of fractions of one, the undeformed
+    lattice (every face vertical or level) and FP16 lattices, whose flat
+    tetrahedra take FP64. A cell's parts are rounded to 2^-28 of the mean cell
+    and come from heights good to 2^-40: 1e-5 of max(cell, mean)."""
+    from paper_1208_3206_gb300.render import Renderer
+    r = Renderer()
+    d = lattice(N, lam, 4) if lam > 0 else np.zeros((N ** 3, 3))
+    if half:
+        p = fp16_offsets(d, N)
+        ref_pos = decoded(p, N)
+    else:
+        if lam == 0:
+            d = d + np.array([0.0123, 0.0077, 0.0031])  # columns off the faces
+        p = ref_pos = wrapped(d, N, 1.0)
+    r.build_tets(torch.from_numpy(p).cuda(), N)
+    grid = r.resample(n, weight)
+    again = r.resample(n, weight)
+    r.sync()
+    ref = oracle.resample(ref_pos, N, n, weight)
+    got = grid.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0 / n))
+    assert torch.equal(grid, again)
