@@ -813,8 +813,7 @@ lt_status lt_render_area(lt_ctx* ctx, const lt_camera* cam, int snapshot, float*
   LT_CUDA(cudaMemcpyAsync(ctx->d_frame_cen, ctx->h_frames, sizeof(FrameDev), cudaMemcpyHostToDevice, s));
   LT_CUDA(cudaMemsetAsync(&ctx->d_ctr->area_pairs, 0, 2 * sizeof(unsigned long long), s));
   // the fixed-point unit is the frame's: 2^-frac_bits of its mean column density
-  LT_CUDA(lt::launch_area(ctx->L, ctx->d_frame_cen, cam->W, cam->H, F.m_tet, F.unit, ctx->d_cacc, d_image, ctx->d_ctr,
-                          s));
+  LT_CUDA(lt::launch_area(ctx->L, F, ctx->d_frame_cen, ctx->d_cacc, d_image, ctx->d_ctr, s));
   LT_CUDA(cudaStreamSynchronize(s));
   return LT_OK;
 }

@@ -104,8 +104,8 @@ cudaError_t launch_fixed_finalize(const unsigned long long* d_acc, long long np,
                                   const FrameDev* d_frame, float* d_out, cudaStream_t s);
 
 // ---- lt_area.cu: area-averaged pixels of one orthographic frame.
-cudaError_t launch_area(const Lattice& L, const FrameDev* d_frame, int W, int H, double m_tet, double unit,
-                        unsigned long long* d_acc, float* d_out, DevCounters* ctr, cudaStream_t s);
+cudaError_t launch_area(const Lattice& L, const FrameDev& F, const FrameDev* d_frame, unsigned long long* d_acc, float* d_out,
+                        DevCounters* ctr, cudaStream_t s);
 
 // ---- lt_backward.cu
 cudaError_t launch_backward(const Lattice& L, const FrameDev* d_frames, long long stride, int n_frames, int n_snap,

@@ -238,3 +238,29 @@ def test_resample_forms(N, n, lam, half, weight):
     got = grid.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0 / n))
     assert torch.equal(grid, again)
+
+
+@pytest.mark.parametrize("N,W,H,kind,lam", [(1, 5, 9, "z", 0.5), (2, 64, 64, "z", 1.0), (4, 300, 210, "z", 2.0), (9, 31, 3, "z", 3.0),
+                                            (24, 20, 20, "z", 3.0), (16, 90, 70, "oblique", 4.0), (6, 41, 37, "z", 0.0)])
+def test_area_stages(N, W, H, kind, lam):
+    """Area-averaged pixels: tetrahedra of thousands of pixels and of fractions
+    of one (squares that hold a whole hull, over several rays, over one, inside
+    one sector), the undeformed lattice (apexes on hull vertices and edges).
+    Lines are good to 2^-24 of a pixel and hulls are 0.05 pixels wide at least
+    in FP32, so a tetrahedron's share is good to about 1e-5 and the pixel to
+    1e-5 of max(pixel, mean)."""
+    from paper_1208_3206_gb300.render import Renderer
+    r = Renderer()
+    d = lattice(N, lam, 6) if lam > 0 else np.zeros((N ** 3, 3))
+    p = wrapped(d, N, 1.0)
+    cam = view(W, H, "z")
+    if kind == "oblique":
+        cam = dict(type="ortho", W=W, H=H, fwd=(1.0, 2.0, 2.5), up=(0, 0, 1), lo=(-0.4, -0.6), hi=(0.8, 0.7), wrap=False)
+    r.build_tets(torch.from_numpy(p).cuda(), N)
+    img = r.render_area(cam)
+    again = r.render_area(cam)
+    r.sync()
+    ref = oracle.render_area(p, N, cam)
+    got = img.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
+    assert torch.equal(img, again)
