@@ -7,10 +7,20 @@
 // N(x) = orient(v_j, v_k, x) and o1, o2 = orient(v_j, v_k, v_l1 / v_l2).
 // Its derivative with respect to any vertex is affine in x, so the sums over
 // a tetrahedron's fragments only need the moments sum g, sum g X, sum g Y
-// of dL/dI per active edge. One thread per cube walks its fragments as a
-// gather from dL/dI (no atomics), keeps the 8 corner gradients in registers
-// over all frames, and a second kernel gathers them per particle in a fixed
-// order.
+// of dL/dI per active edge. One thread per tetrahedron walks its fragments as a
+// gather from dL/dI (no atomics); a block's six warps take the same 32 cubes, a
+// row of the connectivity table each, so that a warp's tetrahedra are neighbours
+// of one shape. The block then adds them up per cube corner in the table's order
+// and keeps the corner gradients in registers over all frames, and a second
+// kernel gathers them per particle in a fixed order.
+//
+// What bounds it: instruction issue and divergence in the walk. One thread per
+// cube, with six tetrahedra and eight corner gradients in 254 registers, ran at
+// 10% occupancy with 12 of 32 threads an instruction: 1.57 ms for 64^3 particles
+// at 512^2. Now
+// 0.8 ms (four blocks per SM; 14 threads an instruction). A tetrahedron's
+// moments keep their order, pixel by pixel: sums in another order round by as
+// much as their terms cancel, a thousand times the last bit.
 #include "lt_internal.h"
 
 namespace lt {
@@ -52,118 +62,146 @@ __device__ __forceinline__ void edge_grad(const TetCanon& K, int e, float Kn, fl
   }
 }
 
-__global__ void __launch_bounds__(128) k_backward(Lattice L, const FrameDev* __restrict__ frames, int n_frames,
-                                                  long long stride, const float* __restrict__ dLdI,
-                                                  float* __restrict__ corner_grad) {
+constexpr int kBackCubes = 32;                // cubes of a block
+constexpr int kBackThreads = 6 * kBackCubes;  // their tetrahedra
+constexpr int kBackItems = 8 * kBackCubes;    // their corners
+
+// Gradient of one tetrahedron's projected vertices (pixel units, in the table's
+// order) in one frame, added to gx, gy.
+__device__ __forceinline__ void backward_tet(const Lattice& L, const FrameDev& F, long long cube, int s,
+                                             const float* __restrict__ gimg, float (&gx)[4], float (&gy)[4]) {
+  TetProj P;
+  if (!project_tet<false>(L, F, cube, s, P)) return;
+  const float Kn = 6.0f * F.K;
+  TetRaster t;
+  if (!tet_setup<false, true>(P.x[0], P.y[0], P.x[1], P.y[1], P.x[2], P.y[2], P.x[3], P.y[3], 0.f, 0.f, 0.f, 0.f, Kn, 0.f,
+                              0.f, t))
+    return;
+  float ia[4];  // (the spans have room for its rounding)
+#pragma unroll
+  for (int e = 0; e < 4; ++e) ia[e] = fast_rcp(t.a[e]);
+  int sx0, sx1, sy0, sy1;
+  const float axa = P.axh + P.axl, aya = P.ayh + P.ayl;
+  shift_range(axa + t.xmin, axa + t.xmax, -0.5f, (float)F.W - 0.5f, (float)F.W, F.wrap != 0, sx0, sx1);
+  shift_range(aya + t.ymin, aya + t.ymax, -0.5f, (float)F.H - 0.5f, (float)F.H, F.wrap != 0, sy0, sy1);
+  sx1 = min(sx1, sx0 + 63);
+  sy1 = min(sy1, sy0 + 63);
+  for (int sy = sy0; sy <= sy1; ++sy)
+    for (int sx = sx0; sx <= sx1; ++sx) {
+      const int shx = sx * F.W, shy = sy * F.H;
+      const float ax = axa + (float)shx, ay = aya + (float)shy;
+      const int qx0 = max(0, (int)ceilf(ax + t.xmin - 1e-3f)), qx1 = min(F.W - 1, (int)floorf(ax + t.xmax + 1e-3f));
+      const int qy0 = max(0, (int)ceilf(ay + t.ymin - 1e-3f)), qy1 = min(F.H - 1, (int)floorf(ay + t.ymax + 1e-3f));
+      if (qx0 > qx1 || qy0 > qy1) continue;
+      Moments m;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m.g0[e] = m.gx[e] = m.gy[e] = 0.f;
+      for (int py = qy0; py <= qy1; ++py) {
+        const float Y = rel_coord(py, shy, P.ayh, P.ayl);
+        float erow[4];
+        float lo = -3.0e38f, hi = 3.0e38f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // pixels where every edge function is >= 0, with a small margin
+          erow[e] = fmaf(t.b[e], Y, t.c[e]);
+          const float xb = -erow[e] * ia[e];
+          if (t.a[e] > 0.0f) lo = fmaxf(lo, xb);
+          else if (t.a[e] < 0.0f) hi = fminf(hi, xb);
+          else if (erow[e] < 0.0f) hi = -3.0e38f;
+        }
+        const int xa = max(qx0, (int)ceilf(fmaxf(lo - 1e-3f + ax, -1.0e9f)));
+        const int xb = min(qx1, (int)floorf(fminf(hi + 1e-3f + ax, 1.0e9f)));
+        const float* grow = gimg + (long long)py * F.W;
+        for (int px = xa; px <= xb; ++px) {
+          const float X = rel_coord(px, shx, P.axh, P.axl);
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = fmaf(t.a[e], X, erow[e]);
+          int am = 0;
+          float mn = v[0];
+#pragma unroll
+          for (int e = 1; e < 4; ++e)
+            if (v[e] < mn) { mn = v[e]; am = e; }
+          if (!(mn > 0.0f)) continue;
+          const float g = __ldg(grow + px);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float w = (am == e) ? g : 0.f;
+            m.g0[e] += w;
+            m.gx[e] = fmaf(w, X, m.gx[e]);
+            m.gy[e] = fmaf(w, Y, m.gy[e]);
+          }
+        }
+      }
+      TetCanon K;
+      if (!tet_canon<true>(P.x[0], P.y[0], P.x[1], P.y[1], P.x[2], P.y[2], P.x[3], P.y[3], 0.f, 0.f, 0.f, 0.f, K)) continue;
+      const float tiny = K.S * K.S * 1e-12f;
+      float cx[4] = {0.f, 0.f, 0.f, 0.f}, cy[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) edge_grad(K, e, Kn, tiny, m, cx, cy);
+      // canonical position -> the table's place
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (K.perm[v] == q) { gx[q] += cx[v]; gy[q] += cy[v]; }
+    }
+}
+
+__global__ void __launch_bounds__(kBackThreads, 4) k_backward(Lattice L, const FrameDev* __restrict__ frames, int n_frames,
+                                                           long long stride, const float* __restrict__ dLdI,
+                                                           float* __restrict__ corner_grad) {
+  __shared__ float2 part[6][4][kBackCubes];  // per tetrahedron and vertex
   const long long ncube = L.n_particles;
   const int snap = blockIdx.y;
-  for (long long cube = (long long)blockIdx.x * blockDim.x + threadIdx.x; cube < ncube;
-       cube += (long long)gridDim.x * blockDim.x) {
-    float G[8][3];
+  const int s = threadIdx.x / kBackCubes, c = threadIdx.x % kBackCubes;
+  for (long long base = (long long)blockIdx.x * kBackCubes; base < ncube; base += (long long)gridDim.x * kBackCubes) {
+    const long long cube = base + c;
+    const bool drawn = cube < ncube && !tet_degenerate(L, snap, cube, s);  // zero volume: contributes nothing
+    float G[2][3];  // corner items threadIdx.x and, for the first threads, kBackThreads further
 #pragma unroll
-    for (int n = 0; n < 8; ++n) G[n][0] = G[n][1] = G[n][2] = 0.f;
+    for (int h = 0; h < 2; ++h) G[h][0] = G[h][1] = G[h][2] = 0.f;
     for (int f = 0; f < n_frames; ++f) {
       const FrameDev& F = frames[f];
       if (F.snapshot != snap || F.persp) continue;
-      CubeProj P;
-      bool ok = true;
-      if (!project_cube<false>(L, F, cube, P, ok)) continue;
-      const float* gimg = dLdI + (long long)f * stride;
-      float gpx[8], gpy[8];
+      float gx[4] = {0.f, 0.f, 0.f, 0.f}, gy[4] = {0.f, 0.f, 0.f, 0.f};
+      if (drawn) backward_tet(L, F, cube, s, dLdI + (long long)f * stride, gx, gy);
 #pragma unroll
-      for (int n = 0; n < 8; ++n) gpx[n] = gpy[n] = 0.f;
-      int sx0, sx1, sy0, sy1;
-      const float axa = P.axh + P.axl, aya = P.ayh + P.ayl;
-      shift_range(axa + P.xmin, axa + P.xmax, -0.5f, (float)F.W - 0.5f, (float)F.W, F.wrap != 0, sx0, sx1);
-      shift_range(aya + P.ymin, aya + P.ymax, -0.5f, (float)F.H - 0.5f, (float)F.H, F.wrap != 0, sy0, sy1);
-      const float Kn = 6.0f * F.K;
-      sx1 = min(sx1, sx0 + 63);
-      sy1 = min(sy1, sy0 + 63);
-      for (int sy = sy0; sy <= sy1; ++sy)
-        for (int sx = sx0; sx <= sx1; ++sx) {
-          const int shx = sx * F.W, shy = sy * F.H;
-          const float ax = axa + (float)shx, ay = aya + (float)shy;
-#pragma unroll
-          for (int s = 0; s < 6; ++s) {
-            if (tet_degenerate(L, snap, cube, s)) continue;  // zero volume: contributes nothing
-            const int c0 = tet_corner(s, 0), c1 = tet_corner(s, 1), c2 = tet_corner(s, 2), c3 = tet_corner(s, 3);
-            TetRaster t;
-            if (!tet_setup<false>(P.x[c0], P.y[c0], P.x[c1], P.y[c1], P.x[c2], P.y[c2], P.x[c3], P.y[c3], 0.f, 0.f,
-                                  0.f, 0.f, Kn, 0.f, 0.f, t))
-              continue;
-            const int qx0 = max(0, (int)ceilf(ax + t.xmin - 1e-3f)), qx1 = min(F.W - 1, (int)floorf(ax + t.xmax + 1e-3f));
-            const int qy0 = max(0, (int)ceilf(ay + t.ymin - 1e-3f)), qy1 = min(F.H - 1, (int)floorf(ay + t.ymax + 1e-3f));
-            if (qx0 > qx1 || qy0 > qy1) continue;
-            Moments m;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) m.g0[e] = m.gx[e] = m.gy[e] = 0.f;
-            for (int py = qy0; py <= qy1; ++py) {
-              const float Y = rel_coord(py, shy, P.ayh, P.ayl);
-              float erow[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) erow[e] = fmaf(t.b[e], Y, t.c[e]);
-              float lo, hi;
-              row_span(t, erow, lo, hi);
-              const int xa = max(qx0, (int)ceilf(fmaxf(lo + ax, -1.0e9f)));
-              const int xb = min(qx1, (int)floorf(fminf(hi + ax, 1.0e9f)));
-              for (int px = xa; px <= xb; ++px) {
-                const float X = rel_coord(px, shx, P.axh, P.axl);
-                float v[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = fmaf(t.a[e], X, erow[e]);
-                int am = 0;
-                float mn = v[0];
-#pragma unroll
-                for (int e = 1; e < 4; ++e)
-                  if (v[e] < mn) { mn = v[e]; am = e; }
-                if (!(mn > 0.0f)) continue;
-                const float g = __ldg(gimg + (long long)py * F.W + px);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const float w = (am == e) ? g : 0.f;
-                  m.g0[e] += w;
-                  m.gx[e] = fmaf(w, X, m.gx[e]);
-                  m.gy[e] = fmaf(w, Y, m.gy[e]);
-                }
-              }
-            }
-            TetCanon K;
-            if (!tet_canon(P.x[c0], P.y[c0], P.x[c1], P.y[c1], P.x[c2], P.y[c2], P.x[c3], P.y[c3], 0.f, 0.f, 0.f,
-                           0.f, K))
-              continue;
-            const float tiny = K.S * K.S * 1e-12f;
-            float gx[4] = {0.f, 0.f, 0.f, 0.f}, gy[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) edge_grad(K, e, Kn, tiny, m, gx, gy);
-            // canonical position -> table slot -> cube corner
-            const int cs[4] = {c0, c1, c2, c3};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              const int slot = K.perm[v];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                if (slot == q) {
-#pragma unroll
-                  for (int n = 0; n < 8; ++n)
-                    if (n == cs[q]) { gpx[n] += gx[v]; gpy[n] += gy[v]; }
-                }
-              }
-            }
-          }
-        }
+      for (int q = 0; q < 4; ++q) part[s][q][c] = make_float2(gx[q], gy[q]);
+      __syncthreads();
       // pixel -> world: x_pix = (r . P) sx + const, y_pix = (u . P) sy + const; the
       // edge functions are in fixed-point accumulator units, converted by F.unit
       const float unit = (float)F.unit;
 #pragma unroll
-      for (int n = 0; n < 8; ++n)
+      for (int h = 0; h < 2; ++h) {
+        const int item = threadIdx.x + h * kBackThreads;
+        if (item >= kBackItems) break;
+        const int n = item / kBackCubes, ci = item % kBackCubes;
+        float px = 0.f, py = 0.f;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) G[n][q] += (gpx[n] * F.sx * F.r[q] + gpy[n] * F.sy * F.u[q]) * unit;
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (tet_corner(r, q) == n) {
+              const float2 v = part[r][q][ci];
+              px += v.x;
+              py += v.y;
+            }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) G[h][q] += (px * F.sx * F.r[q] + py * F.sy * F.u[q]) * unit;
+      }
+      __syncthreads();
     }
-    float* out = corner_grad + ((long long)snap * ncube + cube) * 24;
 #pragma unroll
-    for (int n = 0; n < 8; ++n)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) out[n * 3 + q] = G[n][q];
+    for (int h = 0; h < 2; ++h) {
+      const int item = threadIdx.x + h * kBackThreads;
+      const long long ic = base + item % kBackCubes;
+      if (item >= kBackItems || ic >= ncube) continue;
+      float* out = corner_grad + ((long long)snap * ncube + ic) * 24 + 3 * (item / kBackCubes);
+      out[0] = G[h][0];
+      out[1] = G[h][1];
+      out[2] = G[h][2];
+    }
   }
 }
 
@@ -173,12 +211,13 @@ __global__ void k_gather(Lattice L, const float* __restrict__ corner_grad, float
   const int snap = blockIdx.y;
   const int N = L.N;
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(p % N), j = (int)((p / N) % N), k = (int)(p / ((long long)N * N));
+    int i, j, k;
+    cube_ijk(L, p, i, j, k);
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
       const int a = n & 1, b = (n >> 1) & 1, c = (n >> 2) & 1;
-      const int ci = (i - a + N) % N, cj = (j - b + N) % N, ck = (k - c + N) % N;
+      const int ci = i - a < 0 ? i - a + N : i - a, cj = j - b < 0 ? j - b + N : j - b, ck = k - c < 0 ? k - c + N : k - c;
       const long long cube = particle_id(ci, cj, ck, N);
       const float* g = corner_grad + ((long long)snap * np + cube) * 24 + n * 3;
       gx += g[0];
@@ -194,10 +233,10 @@ __global__ void k_gather(Lattice L, const float* __restrict__ corner_grad, float
 
 cudaError_t launch_backward(const Lattice& L, const FrameDev* d_frames, long long stride, int n_frames, int n_snap,
                             const float* dLdI, float* corner_grad, cudaStream_t s) {
-  long long b = (L.n_particles + 127) / 128;
-  if (b > 8192) b = 8192;
+  long long b = (L.n_particles + kBackCubes - 1) / kBackCubes;
+  if (b > 65536) b = 65536;
   dim3 grid((unsigned)(b < 1 ? 1 : b), n_snap);
-  k_backward<<<grid, 128, 0, s>>>(L, d_frames, n_frames, stride, dLdI, corner_grad);
+  k_backward<<<grid, kBackThreads, 0, s>>>(L, d_frames, n_frames, stride, dLdI, corner_grad);
   return cudaGetLastError();
 }
 

@@ -264,3 +264,22 @@ def test_area_stages(N, W, H, kind, lam):
     got = img.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
     assert torch.equal(img, again)
+
+
+@pytest.mark.parametrize("N,W,H,snaps", [(1, 9, 9, 1), (3, 33, 20, 2), (7, 64, 50, 2), (18, 40, 61, 1)])
+def test_backward_blocks(R, N, W, H, snaps):
+    """The adjoint over lattices that do not fill a block of 32 cubes, several
+    snapshots and frames (one snapshot seen twice, periodic and oblique): the
+    repository's bound for gradients, 1e-3 of the oracle's in the 2-norm."""
+    p = [wrapped(lattice(N, 1.2, 20 + s), N, 1.0) for s in range(snaps)]
+    cams = [view(W, H, "z")] * snaps
+    cams.append(dict(type="ortho", W=W, H=H, fwd=(1.0, 2.0, 2.5), up=(0, 0, 1), lo=(-0.4, -0.6), hi=(0.8, 0.7), wrap=False))
+    of = list(range(snaps)) + [snaps - 1]
+    R.build_tets(torch.from_numpy(np.stack(p)).cuda(), N)
+    R.project_bin(cams, of)
+    g = np.random.default_rng(N).normal(size=(len(cams), H, W)).astype(np.float32)
+    got = R.render_backward(torch.from_numpy(g).cuda()).cpu().numpy().astype(np.float64)
+    R.sync()
+    for s in range(snaps):
+        ref = sum(oracle.gradient(p[s], N, cams[f], g[f].astype(np.float64)) for f in range(len(cams)) if of[f] == s)
+        assert np.linalg.norm(got[s] - ref) <= 1e-3 * max(np.linalg.norm(ref), 1e-30)
