@@ -66,6 +66,7 @@ struct lt_ctx {
   unsigned long long* d_frag = nullptr;
   size_t frag_cap = 0;
   unsigned long long* h_u64 = nullptr;  // pinned scratch
+  cudaEvent_t sized = nullptr;          // the lists' size has reached h_u64
   // zero-volume tetrahedra: one bit per tetrahedron, a byte per (snapshot, cube)
   unsigned char* d_degen = nullptr;
   size_t degen_cap = 0;
@@ -373,29 +374,42 @@ lt_status grow_zeroed(lt_ctx* ctx, T** p, size_t* cap, size_t n, cudaStream_t s)
   return LT_OK;
 }
 
+// The scatter into the lists (cursors at zero) and the work list.
+lt_status scatter_launches(lt_ctx* ctx, cudaStream_t s, bool latch) {
+  LT_CUDA(lt::launch_bin_scatter(ctx->L, ctx->d_frames, ctx->n_frames, ctx->d_off, ctx->d_cursor, ctx->d_list,
+                                 ctx->list_cap, latch, ctx->d_desc, ctx->d_ctr, s));
+  // (the cursors are spent: their array takes the tiles' slots)
+  LT_CUDA(lt::launch_worklist(ctx->d_off, ctx->n_tiles, work_target(ctx), ctx->d_hist, ctx->d_work, ctx->d_cursor, s));
+  return LT_OK;
+}
+
 // Launches of the bin pass after the frames are on the device.
 lt_status bin_launches(lt_ctx* ctx, cudaStream_t s, bool allow_sync) {
   const long long n = ctx->n_tiles;
   LT_CUDA(cudaMemsetAsync(ctx->d_count, 0, sizeof(unsigned) * n, s));
   LT_CUDA(lt::launch_bin_count(ctx->L, ctx->d_frames, ctx->n_frames, ctx->d_count, ctx->d_desc, ctx->d_ctr, s));
-  LT_CUDA(lt::launch_scan(ctx->d_count, n, ctx->d_off, ctx->d_scan_tmp, s));
+  LT_CUDA(lt::launch_scan(ctx->d_count, n, ctx->d_off, ctx->d_cursor, ctx->d_scan_tmp, s));
   if (allow_sync) {
     LT_CUDA(cudaMemcpyAsync(ctx->h_u64, ctx->d_off + n, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    LT_CUDA(cudaStreamSynchronize(s));
-    const unsigned long long total = ctx->h_u64[0];
-    ctx->entries = total;
-    if (total > ctx->list_cap) {
-      size_t cap = ctx->list_cap;
-      lt_status st = grow_c(ctx, &ctx->d_list, &cap, (size_t)(total + total / 8 + 1024));
-      if (st != LT_OK) return st;
-      ctx->list_cap = cap;
-    }
+    LT_CUDA(cudaEventRecord(ctx->sized, s));
   }
-  LT_CUDA(cudaMemsetAsync(ctx->d_cursor, 0, sizeof(unsigned) * n, s));
-  LT_CUDA(lt::launch_bin_scatter(ctx->L, ctx->d_frames, ctx->n_frames, ctx->d_off, ctx->d_cursor, ctx->d_list,
-                                 ctx->list_cap, ctx->d_desc, ctx->d_ctr, s));
-  // (the cursors are spent: their array takes the tiles' slots)
-  LT_CUDA(lt::launch_worklist(ctx->d_off, n, work_target(ctx), ctx->d_hist, ctx->d_work, ctx->d_cursor, s));
+  // the rest goes ahead with the lists as they are while the host waits for
+  // their size; where they turn out too small it is done again after growing
+  // them (a captured pass cannot, and latches what does not fit)
+  lt_status st = scatter_launches(ctx, s, !allow_sync);
+  if (st != LT_OK || !allow_sync) return st;
+  LT_CUDA(cudaEventSynchronize(ctx->sized));
+  const unsigned long long total = ctx->h_u64[0];
+  ctx->entries = total;
+  if (total > ctx->list_cap) {
+    size_t cap = ctx->list_cap;
+    LT_CUDA(cudaStreamSynchronize(s));
+    st = grow_c(ctx, &ctx->d_list, &cap, (size_t)(total + total / 8 + 1024));
+    ctx->list_cap = cap;  // (0 without memory for them)
+    if (st != LT_OK) return st;
+    LT_CUDA(cudaMemsetAsync(ctx->d_cursor, 0, sizeof(unsigned) * n, s));
+    return scatter_launches(ctx, s, true);
+  }
   return LT_OK;
 }
 
@@ -574,6 +588,7 @@ lt_status lt_create(lt_ctx** out, const lt_config* cfg) {
   if (cudaMalloc((void**)&ctx->d_ctr, sizeof(DevCounters)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_ctr, sizeof(DevCounters)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->h_u64, 64 * sizeof(unsigned long long)) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ctx->sized, cudaEventDisableTiming) != cudaSuccess ||
       cudaMalloc((void**)&ctx->d_hist, lt::kHistWords * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     lt_destroy(ctx);
@@ -616,6 +631,7 @@ void lt_destroy(lt_ctx* ctx) {
   cudaFree(ctx->d_degen);
   if (ctx->h_ctr) cudaFreeHost(ctx->h_ctr);
   if (ctx->h_u64) cudaFreeHost(ctx->h_u64);
+  if (ctx->sized) cudaEventDestroy(ctx->sized);
   if (ctx->h_frames) cudaFreeHost(ctx->h_frames);
   delete ctx;
 }
@@ -846,8 +862,9 @@ lt_status lt_graph_build(lt_ctx* ctx, const lt_camera* cams, int n_frames, const
   const unsigned long long want = ctx->entries + ctx->entries / 4 + 4096;
   if (want > ctx->list_cap) {
     size_t cap = ctx->list_cap;
-    if ((st = grow(&ctx->d_list, &cap, (size_t)want)) != LT_OK) return st;
+    st = grow(&ctx->d_list, &cap, (size_t)want);
     ctx->list_cap = cap;
+    if (st != LT_OK) return st;
     // the reallocation dropped the lists just built: bin again, so that direct
     // renders of these frames stay valid
     if ((st = bin_launches(ctx, s, true)) != LT_OK) return st;

@@ -17,12 +17,14 @@ cudaError_t launch_build_tets(const Lattice& L, int n_snap, double m, float* rho
 // count pass and read by the scatter
 cudaError_t launch_bin_count(const Lattice& L, const FrameDev* d_frames, int n_frames, unsigned* d_count,
                              unsigned* d_desc, DevCounters* ctr, cudaStream_t s);
-cudaError_t launch_scan(const unsigned* d_count, long long n, unsigned long long* d_off, unsigned long long* d_tmp,
-                        cudaStream_t s);
+// (also zeroes d_cursor, n entries)
+cudaError_t launch_scan(const unsigned* d_count, long long n, unsigned long long* d_off, unsigned* d_cursor,
+                        unsigned long long* d_tmp, cudaStream_t s);
 size_t scan_tmp_words(long long n);
 cudaError_t launch_bin_scatter(const Lattice& L, const FrameDev* d_frames, int n_frames,
                                const unsigned long long* d_off, unsigned* d_cursor, unsigned* d_list,
-                               unsigned long long capacity, unsigned* d_desc, DevCounters* ctr, cudaStream_t s);
+                               unsigned long long capacity, bool latch, unsigned* d_desc, DevCounters* ctr,
+                               cudaStream_t s);
 // Work list of the raster: every tile's list in chunks of work_chunk() cubes,
 // longest first; d_slot receives the slot of each tile that has several.
 cudaError_t launch_worklist(const unsigned long long* d_off, long long n_tiles, unsigned work_target, unsigned* d_hist,
@@ -33,10 +35,16 @@ constexpr int kWorkChunkBits = 20;
 constexpr int kBuckets = 34;                  // list lengths by log2
 constexpr int kHistItems = 2 * kBuckets;      // d_hist: number of items, then of slots
 constexpr int kHistWords = 2 * kBuckets + 2;
-// Items a CTA gets on average beyond one per tile: enough that the longest
-// first leave the CTAs within a few percent of each other at the end.
-constexpr unsigned kItemsPerCta = 16;
-constexpr unsigned long long kMinChunk = 128;  // one batch of 16 cubes for each of 8 warps
+// Items beyond one per tile, per resident pair of CTAs on an SM: enough that
+// the longest first leave the CTAs close to each other at the end, and not so
+// many that a tile's parts cost more to put together than they balance (16
+// instead of 6: a fitting step of 64^3 at 512^2 1.73 ms, not 1.53; 2: a
+// perspective frame of 128^3 2.71, not 2.35).
+constexpr unsigned kItemsPerCta = 6;
+// Least cubes of an item, a batch of 16 or two for each of its 8 warps: below,
+// a tile's clearing, barriers and sums cost more than the cubes (a frame of
+// 32^3 at 256^2: 230 us at 64, 182 at 128, 170 at 192).
+constexpr unsigned long long kMinChunk = 192;
 
 // Cubes per item when `total` list entries are spread over work_target
 // (CTAs x kItemsPerCta) items: the lists then make at most work_target items

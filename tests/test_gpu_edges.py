@@ -184,6 +184,28 @@ def test_raster_items(kind, N, W, H, tile, frac_bits):
     assert torch.equal(r.render_tiles()[0], img[0])
 
 
+@pytest.mark.parametrize("W,H,tile", [(1024, 1024, 16), (1040, 1024, 16), (512, 512, 8), (64, 64, 64)])
+def test_worklist_forms(W, H, tile):
+    """4096 tiles (the work list of one block), more, and as many frames as make
+    more; lists that grow from nothing, from those of fewer frames and of a
+    smaller lattice, and that are too large. Sums are fixed-point: bit for bit."""
+    from paper_1208_3206_gb300.render import Renderer
+    cam = view(W, H, "persp")
+    small, large = wrapped(lattice(8, 1.0, 5), 8, 1.0), wrapped(lattice(24, 2.0, 3), 24, 1.0)
+    images = []
+    for order in ([1], [1, 3], [3, 1], [0, 1]):
+        r = Renderer(tile=tile)
+        for frames in order:
+            r.build_tets(torch.from_numpy(large if frames else small).cuda(), 24 if frames else 8)
+            r.project_bin([cam] * max(frames, 1))
+            img = r.render_tiles()
+        r.sync()
+        images += [x for x in img] if frames else []
+    assert images[0].sum() > 0
+    for x in images[1:]:
+        assert torch.equal(x, images[0])
+
+
 @pytest.mark.parametrize("N,W,H,kind,lam,half", [(1, 9, 7, "z", 0.5, False), (3, 40, 33, "z", 1.0, False), (13, 300, 7, "z", 2.0, False),
                                                  (49, 61, 50, "z", 3.0, False), (50, 64, 48, "persp", 2.0, False),
                                                  (16, 256, 256, "persp", 4.0, False), (20, 90, 80, "z", 6.0, True)])
