@@ -132,34 +132,11 @@ __device__ __forceinline__ int warp_excl_scan(int n, int& total) {
   return incl - n;
 }
 
-// Two FP32 fused multiply-adds in one instruction, each rounded like fmaf.
-__device__ __forceinline__ unsigned long long pack2(float x, float y) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Pixel sums: 64-bit fixed-point integers as two planes of 32-bit words in
-// shared memory (a 32-bit shared atomic is one instruction), addressed by
-// shared-window addresses. Carries into the high word are rare: the low word
+// shared memory (a 32-bit shared atomic is one instruction). Carries into the high word are rare: the low word
 // holds 2^32 units, 16 times the mean column density at the default 28
 // fraction bits.
-__device__ __forceinline__ unsigned smem_add(unsigned addr, unsigned v) {
-  unsigned old;
-  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
-  return old;
-}
-
+//
 // The rest of an add whose low word wrapped, or whose value passes 32 bits (u
 // is then the saturated 2^32 - 1): brings the sum to what adding the whole
 // value gives. A value that cannot be converted (2^63 units or more; it adds

@@ -233,6 +233,24 @@ def test_centroid_blocks(N, W, H, kind, lam, half):
     assert torch.equal(img, again)
 
 
+@pytest.mark.parametrize("frac_bits", [31, 34, 40])
+def test_centroid_peaks(frac_bits):
+    """Pixel sums of finer units than a window's 32-bit words hold: a few of
+    the splats, most and all of them go to the image directly. Against the sums
+    at the default 28 bits: a unit is 2^-28 of the mean, and half units of either
+    sign from 10^5 splats in a pixel make 6e-7 of it (the FP32 values are the
+    same on both routes); 1e-5 leaves a factor for the fullest pixel."""
+    from paper_1208_3206_gb300.render import Renderer
+    p = torch.from_numpy(wrapped(lattice(49, 3.0, 9), 49, 1.0)).cuda()
+    images = []
+    for bits in (0, frac_bits):
+        r = Renderer(frac_bits=bits)
+        r.build_tets(p, 49)
+        images.append(r.render_centroids(view(150, 131, "z")))
+        r.sync()
+    assert (images[0] - images[1]).abs().max() <= 1e-5 * images[0].mean()
+
+
 @pytest.mark.parametrize("N,n,lam,half", [(1, 4, 0.5, False), (2, 33, 1.0, False), (5, 1, 1.0, False), (6, 70, 2.0, False),
                                           (11, 24, 3.0, False), (33, 8, 3.0, False), (16, 40, 4.0, True), (12, 31, 0.0, False)])
 @pytest.mark.parametrize("weight", ["density", "streams"])
