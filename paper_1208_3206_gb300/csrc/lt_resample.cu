@@ -36,14 +36,17 @@
 // What bounds it: with the planes, the intervals and their pieces in FP64 the
 // FP64 pipe took 148 ms for 128^3 particles onto 512^3 cells (1.6e8 intervals,
 // 3.0e8 pieces), 19 of them the setup, done once for each tile of columns that a
-// tetrahedron touched. Now 9.5 ms for the call, of which the
-// grid's clearing and conversion are 0.45; the kernel issues in 55% of its slots.
+// tetrahedron touched. Now 8.6 ms for the call, of which the
+// grid's clearing and conversion are 0.45; the kernel issues in about 60% of its
+// slots, and waits for global memory most in the others.
 #include "lt_ff.cuh"
 #include "lt_internal.h"
 
 namespace lt {
 
-constexpr int kResampleThreads = 128;
+// Two warps: they are done at different times, and the shared memory of a small
+// block goes on to the next one sooner (blocks of four warps 9.45 ms, of one 8.65).
+constexpr int kResampleThreads = 64;
 constexpr int kZBits = 42;  // fraction bits of a height in cells
 constexpr long long kZOne = 1LL << kZBits;
 
