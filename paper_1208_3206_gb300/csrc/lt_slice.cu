@@ -27,10 +27,11 @@
 //
 // What bounds it: with the corners of every cube in FP64 and one thread per
 // cube walking its points, the FP64 pipe took 29.4 ms for 256^3 particles and
-// 2048^2 points; now 1.18 ms, of which the FP32 scan of all cubes is 0.41 (its
-// 16-byte particles alone 0.04), the FP64 setup at the plane 0.6, the points
-// 0.15. Five resident blocks (96 registers) hide the scan's loads; at three
-// (148 registers) the kernel took 1.35 ms.
+// 2048^2 points; now 1.1 ms, of which the FP32 scan of all cubes is about 0.4
+// (its 16-byte particles alone 0.04), the FP64 setup at the plane 0.5, the points
+// 0.15. Six resident blocks, what shared memory holds, hide the scan's loads (72
+// registers, cut for seven; 80, cut for six, are 3% slower): five (96 registers)
+// took 1.19 ms, three (148) 1.35, blocks of 64 threads 1.22.
 #include <math.h>
 
 #include "lt_internal.h"
@@ -130,7 +131,7 @@ __device__ __forceinline__ void slice_add(const SliceArgs& a, long long bw, long
   atomicAdd(&a.ctr->range_overflow, 1ull);
 }
 
-__global__ void __launch_bounds__(kSliceThreads, 5) k_slice(SliceArgs a) {
+__global__ void __launch_bounds__(kSliceThreads, 7) k_slice(SliceArgs a) {
   __shared__ SliceTet tets[kSliceThreads];
   __shared__ unsigned short list[6 * kSliceCubes];  // 6 x cube of the block + s
   __shared__ int n_list;
