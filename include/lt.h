@@ -249,8 +249,9 @@ lt_status lt_render_backward(lt_ctx* ctx, const float* d_dL_dimage, float* d_dL_
  * line against the four face planes, to about 2^-40 of a cell; the cells are summed as
  * 64-bit fixed-point integers (2^-frac_bits of the mean cell), so the grid
  * is bitwise reproducible. Tetrahedra with V == 0 contribute nothing.
- * Asynchronous; leaves the bins of the last lt_project_bin untouched; keeps an
- * n^3 array of 64-bit cells in the context.
+ * Asynchronous, without bins of its own; render or count afterwards only after
+ * a new lt_project_bin (LT_ERR_STATE). Keeps an n^3 array of 64-bit cells in
+ * the context.
  * Errors: LT_ERR_STATE (no lt_build_tets), LT_ERR_ARG (null d_grid, n < 1 or
  * n > 2048, unknown weight, snapshot out of range), LT_ERR_NOMEM; a cell
  * leaving the fixed-point range latches LT_ERR_RANGE.

@@ -60,6 +60,7 @@ struct lt_ctx {
   unsigned* d_desc = nullptr;  // per (frame, cube) tile descriptors of the bin pass (null above the budget)
   size_t desc_cap = 0;
   bool binned = false;
+  bool resampled = false;  // since the frames were binned: renders and counts want them binned again
   // counters
   DevCounters* d_ctr = nullptr;
   DevCounters* h_ctr = nullptr;  // pinned
@@ -492,6 +493,7 @@ lt_status project_bin_impl(lt_ctx* ctx, const lt_camera* cams, int n_frames, con
   ctx->any_persp = any_persp;
   ctx->n_tiles = n_tiles;
   ctx->binned = true;
+  ctx->resampled = false;
   return bin_launches(ctx, s, !is_capturing(s));
 }
 
@@ -690,7 +692,7 @@ lt_status lt_project_bin(lt_ctx* ctx, const lt_camera* cams, int n_frames, const
 
 lt_status lt_render_tiles(lt_ctx* ctx, float* d_image, double* d_mass, lt_stream stream) {
   if (!ctx || !d_image) return LT_ERR_ARG;
-  if (!ctx->binned) return LT_ERR_STATE;
+  if (!ctx->binned || ctx->resampled) return LT_ERR_STATE;
   return render_impl(ctx, d_image, d_mass, (cudaStream_t)stream);
 }
 
@@ -713,7 +715,7 @@ lt_status lt_render_atomic(lt_ctx* ctx, const lt_camera* cams, int n_frames, con
 
 lt_status lt_count_fragments(lt_ctx* ctx, long long* h_counts, lt_stream stream) {
   if (!ctx || !h_counts) return LT_ERR_ARG;
-  if (!ctx->binned) return LT_ERR_STATE;
+  if (!ctx->binned || ctx->resampled) return LT_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
   lt_status st = grow(&ctx->d_frag, &ctx->frag_cap, (size_t)ctx->n_frames);
   if (st != LT_OK) return st;
@@ -774,6 +776,7 @@ lt_status lt_resample(lt_ctx* ctx, int n, int weight, int snapshot, float* d_gri
   lt_status st;
   const size_t cells = (size_t)n * n * n;
   if ((st = grow(&ctx->d_racc, &ctx->racc_cap, cells)) != LT_OK) return st;
+  ctx->resampled = true;
   const double box = ctx->L.box, gs = box / n;
   const int N = ctx->L.N;
   const double m_tet = ctx->total_mass / (6.0 * (double)N * N * N);

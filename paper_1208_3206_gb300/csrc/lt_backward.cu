@@ -17,10 +17,9 @@
 // What bounds it: instruction issue and divergence in the walk. One thread per
 // cube, with six tetrahedra and eight corner gradients in 254 registers, ran at
 // 10% occupancy with 12 of 32 threads an instruction: 1.57 ms for 64^3 particles
-// at 512^2. Now
-// 0.8 ms (four blocks per SM; 14 threads an instruction). A tetrahedron's
-// moments keep their order, pixel by pixel: sums in another order round by as
-// much as their terms cancel, a thousand times the last bit.
+// at 512^2. Now 0.75 ms (four blocks per SM; 14 threads an instruction). A
+// tetrahedron's moments keep their order, pixel by pixel: sums in another order
+// round by as much as their terms cancel, a thousand times the last bit.
 #include "lt_internal.h"
 
 namespace lt {

@@ -198,13 +198,14 @@ class Renderer:
         """Resampling of one registered snapshot onto a periodic n^3 grid
         (float32 [n][n][n], index [c][b][a]): per cell, q dl along its
         central line in z inside its slab, q = rho ("density") or 1
-        ("streams")."""
+        ("streams"). Rendering or counting afterwards takes a new project_bin."""
         w = {"density": 0, "streams": 1}[weight]
         if out is None:
             out = torch.empty((n, n, n), dtype=torch.float32, device="cuda")
         if out.dtype != torch.float32 or not out.is_cuda or out.numel() != n ** 3 or not out.is_contiguous():
             raise ValueError("out must be a contiguous float32 CUDA tensor with n^3 elements")
         check("lt_resample", self._lib.lt_resample(self._h, int(n), w, int(snapshot), _ptr(out), _stream()))
+        self._cams = []
         return out
 
     # -- lt_slice

@@ -280,6 +280,25 @@ def test_resample_forms(N, n, lam, half, weight):
     assert torch.equal(grid, again)
 
 
+def test_resample_between_bin_and_render():
+    """A grid needs no bins, but as ever the frames are binned again before they
+    are rendered or counted; the adjoint of the binned frames stands."""
+    from paper_1208_3206_gb300.render import Renderer
+    N, cam = 8, view(32, 24, "z")
+    r = Renderer()
+    r.build_tets(torch.from_numpy(wrapped(lattice(N, 1.0, 2), N, 1.0)).cuda(), N)
+    r.project_bin([cam])
+    img = r.render_tiles()
+    grad = r.render_backward(2.0 * img).clone()
+    r.resample(16, "density")
+    with pytest.raises(Exception):
+        r.render_tiles(img)
+    assert r._lib.lt_render_tiles(r._h, img.data_ptr(), None, None) != 0
+    assert torch.equal(r.render_backward(2.0 * img), grad)
+    r.project_bin([cam])
+    assert torch.equal(r.render_tiles(), img)
+
+
 @pytest.mark.parametrize("N,W,H,kind,lam", [(1, 5, 9, "z", 0.5), (2, 64, 64, "z", 1.0), (4, 300, 210, "z", 2.0), (9, 31, 3, "z", 3.0),
                                             (24, 20, 20, "z", 3.0), (16, 90, 70, "oblique", 4.0), (6, 41, 37, "z", 0.0)])
 def test_area_stages(N, W, H, kind, lam):
