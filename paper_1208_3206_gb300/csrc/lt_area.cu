@@ -207,11 +207,13 @@ __device__ __forceinline__ void keep_from(float p, float q, float iq, float& lo,
   if (q == 0.f && p < 0.f) hi = -1.f;
 }
 
-// Six times the integral of h r dh along a stretch on which h goes from h0 to h1
-// and r from r0 to r1. (The six goes into the divisor at the end: 1/3 and 1/6 in
-// FP32 are both 3e-8 too large, which showed in the frame's mass.)
-__device__ __forceinline__ float stretch(float h0, float h1, float r0, float r1) {
-  return (h1 - h0) * fmaf(2.0f, fmaf(h0, r0, h1 * r1), fmaf(h0, r1, h1 * r0));
+// Six times the integral of h r dh along a stretch on which h goes from h0 to h1,
+// by dh, and r from r0 to r1. (dh from the stretch's length: h1 - h0 would keep
+// the rounding of h far from the hull's edge. The six goes into the divisor at the
+// end: 1/3 and 1/6 in FP32 are both 3e-8 too large, which showed in the frame's
+// mass.)
+__device__ __forceinline__ float stretch(float dh, float h0, float h1, float r0, float r1) {
+  return dh * fmaf(2.0f, fmaf(h0, r0, h1 * r1), fmaf(h0, r1, h1 * r0));
 }
 
 // Integral of the hull line's function h over the part of the unit square in
@@ -247,7 +249,7 @@ __device__ __forceinline__ float sector_part(float ha, float hb, float hc, float
     t1 = fmaxf(t0, t1);
     const float h = fmaf(ha, x0, fmaf(hb, y0, hc)), hs = fmaf(ha, dx, hb * dy);
     const float z = fmaf(za, x0, fmaf(zb, y0, zc)), zs = fmaf(za, dx, zb * dy);
-    sum = t1 > t0 ? sgn * stretch(fmaf(t0, hs, h), fmaf(t1, hs, h), fmaf(t0, zs, z), fmaf(t1, zs, z)) : 0.f;
+    sum = t1 > t0 ? sgn * stretch((t1 - t0) * hs, fmaf(t0, hs, h), fmaf(t1, hs, h), fmaf(t0, zs, z), fmaf(t1, zs, z)) : 0.f;
   }
   // the square's sides: bottom and top along x, left and right along y
   const float iha = __fdividef(1.0f, ha), iza = __fdividef(1.0f, za), ioa = __fdividef(1.0f, oa);
@@ -263,7 +265,7 @@ __device__ __forceinline__ float sector_part(float ha, float hb, float hc, float
     keep_from(zp, zq, along_x ? iza : izb, lo, hi);
     keep_from(op, oq, along_x ? ioa : iob, lo, hi);
     // counter-clockwise: bottom and right forwards, top and left backwards
-    const float part = stretch(fmaf(lo, hq, hp), fmaf(hi, hq, hp), fmaf(lo, zq, zp), fmaf(hi, zq, zp));
+    const float part = stretch((hi - lo) * hq, fmaf(lo, hq, hp), fmaf(hi, hq, hp), fmaf(lo, zq, zp), fmaf(hi, zq, zp));
     if (hi > lo) sum += (along_x ? !far : far) ? part : -part;
   }
   return __fdividef(sum, 6.0f * fmaf(za, hb, -zb * ha));
