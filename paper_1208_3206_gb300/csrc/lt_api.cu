@@ -397,21 +397,23 @@ lt_status bin_launches(lt_ctx* ctx, cudaStream_t s, bool allow_sync) {
   // the rest goes ahead with the lists as they are while the host waits for
   // their size; where they turn out too small it is done again after growing
   // them (a captured pass cannot, and latches what does not fit)
-  lt_status st = scatter_launches(ctx, s, !allow_sync);
+  lt_status st = LT_OK;
+  const bool ahead = !allow_sync || ctx->list_cap > 0;
+  if (ahead) st = scatter_launches(ctx, s, !allow_sync);
   if (st != LT_OK || !allow_sync) return st;
   LT_CUDA(cudaEventSynchronize(ctx->sized));
   const unsigned long long total = ctx->h_u64[0];
   ctx->entries = total;
+  if (ahead && total <= ctx->list_cap) return LT_OK;
   if (total > ctx->list_cap) {
     size_t cap = ctx->list_cap;
     LT_CUDA(cudaStreamSynchronize(s));
     st = grow_c(ctx, &ctx->d_list, &cap, (size_t)(total + total / 8 + 1024));
     ctx->list_cap = cap;  // (0 without memory for them)
     if (st != LT_OK) return st;
-    LT_CUDA(cudaMemsetAsync(ctx->d_cursor, 0, sizeof(unsigned) * n, s));
-    return scatter_launches(ctx, s, true);
   }
-  return LT_OK;
+  if (ahead) LT_CUDA(cudaMemsetAsync(ctx->d_cursor, 0, sizeof(unsigned) * n, s));
+  return scatter_launches(ctx, s, true);
 }
 
 lt_status ensure_tiles(lt_ctx* ctx, long long n, int tile, cudaStream_t s) {
