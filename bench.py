@@ -399,20 +399,11 @@ def run_lt(args, rank: int, world: int):
     return line, (c, pos_np, cams, snaps, gpu_crop, atomic_crops)
 
 
-# FP64 operations the resampling counts (FMA as 2, division as 1): per
-# (tetrahedron, line) interval, four face planes (two FMA and a division
-# each) and four min/max; per piece of an interval in one slab, a max, a min,
-# a subtraction and two multiplications.
-RESAMPLE_FLOPS_PER_INTERVAL = 24
-RESAMPLE_FLOPS_PER_PIECE = 5
-# GB300 FP64 peak (nominal; there is no measured FP64 figure for this machine)
-FP64_PEAK_TFLOPS = 1.25
-
-
 def bench_resample(dev, n: int = 512, reps: int = 3):
     """Time lt_resample of the 128^3 workload (deformation eigenvalue 3) onto
     a periodic n^3 grid, density weighting, with CUDA events; report the
-    (tetrahedron, line) intervals per second and the FP64 roofline."""
+    (tetrahedron, line) intervals per second and the bytes the call cannot do
+    without (positions read, cells written) against the copy bandwidth."""
     import torch
 
     from lt_inputs import ZeldovichField, config
@@ -424,7 +415,7 @@ def bench_resample(dev, n: int = 512, reps: int = 3):
     R = Renderer()
     R.build_tets(pos.to(dev), N)
     grid = torch.empty((n, n, n), dtype=torch.float32, device=dev)
-    R.resample(n, "density", out=grid)  # warm-up (sizes the bins)
+    R.resample(n, "density", out=grid)  # warm-up
     R.sync()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record()
@@ -434,38 +425,23 @@ def bench_resample(dev, n: int = 512, reps: int = 3):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     st = R.get_stats()
-    # its bin pass alone (the same orthographic view of the grid's columns),
-    # to time the resampling kernels without it
-    from lt_inputs import ortho_z
-    b0, b1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    b0.record()
-    for _ in range(reps):
-        R.project_bin([ortho_z(n, n)])
-    b1.record()
-    torch.cuda.synchronize()
-    bin_ms = b0.elapsed_time(b1) / reps
     R.close()
-    kernel_ms = max(ms - bin_ms, 1e-6)
     iv, pc = st["resample_intervals"], st["resample_pieces"]
-    flops = RESAMPLE_FLOPS_PER_INTERVAL * iv + RESAMPLE_FLOPS_PER_PIECE * pc
-    achieved = flops / (kernel_ms * 1e-3) / 1e12
+    hbm, src = copy_peak_gbs()
+    achieved = (16 * N ** 3 + 4 * n ** 3) / (ms * 1e-3) / 1e9
     return {"workload": f"zel128 lattice (12.6M tetrahedra) onto {n}^3 cells, density weighting",
             "ms": ms, "value": iv / (ms * 1e-3), "unit": "intervals/s", "intervals": iv, "pieces": pc,
-            "cells_per_s": n ** 3 / (ms * 1e-3), "bin_ms": bin_ms, "kernel_ms": kernel_ms,
-            "timing": "ms: the whole call, with its bin pass (one host synchronisation); kernel_ms: ms - bin_ms",
-            "roofline": {"bound": "alu", "kernel": "k_resample (FP64 clipping)", "achieved": achieved,
-                         "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s (FP64)", "frac": achieved / FP64_PEAK_TFLOPS,
-                         "counted": f"{RESAMPLE_FLOPS_PER_INTERVAL} FP64 flops per interval + "
-                                    f"{RESAMPLE_FLOPS_PER_PIECE} per slab piece",
-                         "peak_from": "GB300 nominal FP64 rate"}}
+            "cells_per_s": n ** 3 / (ms * 1e-3), "timing": "the whole call",
+            "roofline": {"bound": "memory", "kernel": "k_resample (integer heights) and the grid's clearing and conversion",
+                         "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
+                         "counted": "16 bytes per particle and 4 per cell", "peak_from": src}}
 
 
 # FP32 operations lt_render_area counts per (tetrahedron, pixel) pair: the
-# eight lines (four hull edges, four rays) evaluated at the pixel's corner in
-# float-float (two error-free products, two two-sums and the small terms:
-# 20 operations, FMA as 2), and per pyramid face the corner tests (8); the
-# clip of partly covered squares is not counted.
-AREA_FLOPS_PER_PAIR = 8 * 20 + 4 * 8
+# four hull lines at the pixel's corner (two multiply-adds each) and their
+# largest value over the square (one addition). The lines in float-float, the
+# closed forms and the boundary integrals of the pixels that pass are not counted.
+AREA_FLOPS_PER_PAIR = 4 * 5
 
 
 def bench_area(dev, reps: int = 5):
@@ -506,7 +482,7 @@ def bench_area(dev, reps: int = 5):
             "ms": ms, "value": 1e3 / ms, "unit": "frames/s", "pairs": pairs, "fp64_clip_pairs": p64,
             "pairs_per_s": pairs / (ms * 1e-3), "frame_mass": mass,
             "timing": "the whole call (frame upload, kernel, finalize, one host synchronisation)",
-            "roofline": {"bound": "alu", "kernel": "k_area (float-float lines + FP32 clip)",
+            "roofline": {"bound": "alu", "kernel": "k_area (FP32 reject, closed forms, boundary integrals)",
                          "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak,
                          "counted": f"{AREA_FLOPS_PER_PAIR} FP32 flops per (tetrahedron, pixel) pair",
@@ -581,7 +557,7 @@ def e2e_pipelined(pos, host_pos, img, host_img, N, cams, snaps, cfg, steps, barr
 # DRAM bytes (read + write) of one k_tile launch per frame of the headline
 # workload, from an ncu capture of the kernel built from the sources whose
 # hash is recorded with it; None when the raster has changed since.
-RASTER_TRAFFIC = {"bytes_per_frame": 432438784, "sources_sha16": "d73758b9859dd0d8",
+RASTER_TRAFFIC = {"bytes_per_frame": 574889472, "sources_sha16": "618ac079baa15e99",
                   "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_tile launch, "
                              "python bench.py --one-frame --tile 64 --raster-threads 256 (frame 0), "
                              "scaled by the frames"}
@@ -621,6 +597,19 @@ def fp32_peak_tflops(sms: int):
     except (OSError, ValueError):
         pass
     return sms * 128 * 2 * mhz * 1e6 / 1e12, mhz, src
+
+
+def copy_peak_gbs():
+    """Copy bandwidth of the memory: hbm_gbs of MEASURED_PEAKS.json when it is
+    there, else 6800. Returns (GB/s, where it came from)."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            v = float(json.load(fh).get("hbm_gbs") or 0.0)
+        if v > 0:
+            return v, "hbm_gbs of MEASURED_PEAKS.json (measured copy)"
+    except (OSError, ValueError):
+        pass
+    return 6800.0, "an earlier copy measurement"
 
 
 def central_crop(cam, crop: int):
