@@ -101,8 +101,7 @@ typedef struct {
 
 /* Tuning knobs (lt_autotune fills them; zero fields take defaults). */
 typedef struct {
-  int tile;           /* screen tile edge in pixels: 8, 16, 32 or 64 (default 16; where it is left 0, the
-                         raster takes 32 for FP32 frames of more than 2^20 pixels: lt_stats.tile) */
+  int tile;           /* screen tile edge in pixels: 8, 16, 32 or 64 (default 16) */
   int raster_threads; /* threads per raster CTA: 64..256, multiple of 32 (default 256) */
   int ctas_per_sm;    /* persistent raster CTAs per SM (default: occupancy limit) */
   int frac_bits;      /* fixed-point fraction bits relative to the mean column density sigma, 8..62

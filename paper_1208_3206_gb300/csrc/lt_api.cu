@@ -20,7 +20,6 @@ struct lt_ctx {
   int device = 0;
   int num_sms = 1;
   lt_config cfg{};
-  bool tile_auto = true;  // the caller left the tile edge to the library (see raster_tile)
   // registered lattice
   bool have_lattice = false;
   Lattice L{};
@@ -442,29 +441,11 @@ lt_status ensure_tiles(lt_ctx* ctx, long long n, int tile, cudaStream_t s) {
   return LT_OK;
 }
 
-// Tile edge of the raster where the caller left it open: 32 pixels for frames
-// of more than 2^20. A tetrahedron is set up once for every tile it touches,
-// about (1 + s / T)^2 times for a cell of s pixels, and a span ends at the
-// tile's edge, so larger tiles do less work; but only tiles up to 32 pixels
-// leave shared memory for three CTAs per SM. Measured for tiles of 8, 16, 32
-// and 64, in ms: 128^3 particles at 2048^2 17.6, 10.9, 8.5, 8.7; 16^3 at 1500^2
-// 4.26, 2.24, 1.75, 2.58; 256^3 at 1920 x 1080 in perspective 12.5, 10.6, 9.90,
-// 9.92. Smaller frames would gain as much (128^3 at 1024^2: 4.3 and 3.55), but
-// they are the ones that positions are fitted to, and the gradient of an image
-// loss magnifies the image's last bit a thousand times: they keep the 16 pixels
-// and the bits of the configured tile, as do FP16 lattices (see kTwoStepTile).
-int raster_tile(const lt_ctx* ctx, const lt_camera& c) {
-  if (ctx->L.fmt != LT_POS_F32X4 || (long long)c.W * c.H <= (1LL << 20)) return ctx->cfg.tile;
-  return 32;
-}
-
-// `tile`: tile edge in pixels, or 0 for the context's.
 lt_status project_bin_impl(lt_ctx* ctx, const lt_camera* cams, int n_frames, const int* frame_snapshot,
-                           cudaStream_t s, int tile = 0) {
+                           cudaStream_t s) {
   if (!ctx) return LT_ERR_ARG;
   if (!ctx->have_lattice) return LT_ERR_STATE;
-  if (!cams || n_frames < 1) return LT_ERR_ARG;
-  if (tile == 0) tile = ctx->tile_auto ? raster_tile(ctx, cams[0]) : ctx->cfg.tile;
+  const int tile = ctx->cfg.tile;
   int W, H;
   bool any_persp;
   lt_status st = prepare_frames(ctx, cams, n_frames, frame_snapshot, tile, &W, &H, &any_persp);
@@ -582,7 +563,6 @@ lt_status lt_create(lt_ctx** out, const lt_config* cfg) {
   lt_ctx* ctx = new (std::nothrow) lt_ctx();
   if (!ctx) return LT_ERR_NOMEM;
   ctx->cfg = resolved(cfg ? *cfg : lt_config{});
-  ctx->tile_auto = !cfg || cfg->tile == 0;
   if (cudaGetDevice(&ctx->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
     cudaGetLastError();
@@ -643,7 +623,6 @@ void lt_destroy(lt_ctx* ctx) {
 lt_status lt_set_config(lt_ctx* ctx, const lt_config* cfg) {
   if (!ctx || !cfg || !valid_config(*cfg)) return LT_ERR_ARG;
   ctx->cfg = resolved(*cfg);
-  ctx->tile_auto = cfg->tile == 0;
   return LT_OK;
 }
 
@@ -926,8 +905,6 @@ lt_status lt_autotune(lt_ctx* ctx, const lt_camera* cams, int n_frames, const in
   if (!ctx->have_lattice) return LT_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
   const lt_config base = ctx->cfg;
-  const bool base_auto = ctx->tile_auto;
-  ctx->tile_auto = false;
   const int tiles[] = {16, 32, 64};
   const int threads[] = {128, 256};
   float best_ms = 1e30f;
@@ -966,7 +943,6 @@ lt_status lt_autotune(lt_ctx* ctx, const lt_camera* cams, int n_frames, const in
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   ctx->cfg = result == LT_OK ? best_cfg : base;
-  if (result != LT_OK) ctx->tile_auto = base_auto;
   ctx->binned = false;
   if (best) *best = ctx->cfg;
   return result;

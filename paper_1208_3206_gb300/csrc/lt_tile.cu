@@ -169,15 +169,6 @@ __device__ __forceinline__ void accum_tile(unsigned lo, unsigned plane, float v,
   if (old >= ~u) accum_rest(lo, plane, v, u, old, wraps);
 }
 
-// Tiles up to this edge, and FP16 lattices at any, take a tetrahedron's
-// coordinates relative to its box through the tile's origin, two subtractions
-// with a rounding each. The one-step form rounds less (3.0e-7 against 4.0e-7
-// of a perspective frame), but the gradient of an image loss magnifies the last
-// bit of the image a thousand times, and FP16 lattices hold tetrahedra so flat
-// that the exact evaluation's own rounding shows where a fragment changes to or
-// from it: both keep their fragments and bits as they were (see raster_tile).
-constexpr int kTwoStepTile = 16;
-
 // MIN_CTAS: resident 256-thread CTAs per SM that the register budget is cut for
 // (see tile_min_ctas).
 template <bool ANY_PERSP, bool COUNT, int MIN_CTAS>
@@ -197,7 +188,6 @@ __global__ void __launch_bounds__(256, MIN_CTAS) k_tile(RasterArgs a, unsigned l
   unsigned long long* xq = a.xq + (size_t)blockIdx.x * a.xq_cap;
   const unsigned FULL = 0xffffffffu;
   unsigned long long nfrag = 0;
-  const bool two_step = T <= kTwoStepTile || a.L.fmt != 0;
 
   for (;;) {
     if (threadIdx.x == 0) {
@@ -376,16 +366,14 @@ __global__ void __launch_bounds__(256, MIN_CTAS) k_tile(RasterArgs a, unsigned l
               if (qx0 <= qx1 && qy0 <= qy1) {
                 // the raster form relative to the bounding box's first pixel:
                 // small coordinates keep the round-off of evaluating a x + b y + c
-                // (and with it the exact path's share) small. In one step from the
-                // anchor, so that the tile's place and size do not round; in two
-                // where kTwoStepTile says why
-                const float bx = (float)qx0, by = (float)qy0;
-                const float lx = two_step ? bx : ((float)(tx0 + qx0 - sx * F.W) - an.x) - an.y;
-                const float ly = two_step ? by : ((float)(ty0 + qy0 - sy * F.H) - an.z) - an.w;
-                const float x0 = (two_step ? px[0] - ox : px[0]) - lx, x1 = (two_step ? px[1] - ox : px[1]) - lx;
-                const float x2 = (two_step ? px[2] - ox : px[2]) - lx, x3 = (two_step ? px[3] - ox : px[3]) - lx;
-                const float y0 = (two_step ? py[0] - oy : py[0]) - ly, y1 = (two_step ? py[1] - oy : py[1]) - ly;
-                const float y2 = (two_step ? py[2] - oy : py[2]) - ly, y3 = (two_step ? py[3] - oy : py[3]) - ly;
+                // (and with it the exact path's share) small. In two steps, over
+                // the tile's origin: the difference taken at once from the anchor
+                // rounds a little less, but it changes which fragments of ultra-flat
+                // tetrahedra are evaluated exactly, and with them pixels by up to
+                // 1e-3 of their value
+                const float lx = (float)qx0, ly = (float)qy0;
+                const float x0 = (px[0] - ox) - lx, x1 = (px[1] - ox) - lx, x2 = (px[2] - ox) - lx, x3 = (px[3] - ox) - lx;
+                const float y0 = (py[0] - oy) - ly, y1 = (py[1] - oy) - ly, y2 = (py[2] - oy) - ly, y3 = (py[3] - oy) - ly;
                 float Kn = Kn0;
                 if (persp) Kn = __fdividef(Kn0, pz[0] * pz[1] * pz[2] * pz[3]);
                 const bool set =
