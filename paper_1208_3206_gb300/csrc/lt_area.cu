@@ -236,34 +236,43 @@ __device__ __forceinline__ float sector_part(float ha, float hb, float hc, float
   // where ray z misses the square, z counts from its smallest value there (a
   // constant adds nothing around the piece, and would carry its rounding in)
   zc -= fmaxf(zc + fminf(za, 0.f) + fminf(zb, 0.f), 0.f);
-  float sum;
-  {
-    // ray o, from the point of its line nearest to the square's centre
+  const float iha = __fdividef(1.0f, ha), iza = __fdividef(1.0f, za), ioa = __fdividef(1.0f, oa);
+  const float ihb = __fdividef(1.0f, hb), izb = __fdividef(1.0f, zb), iob = __fdividef(1.0f, ob);
+  // where line o crosses the square's sides: its signs at the corners, of which
+  // rounding cannot make more than two neighbours differ, and its root on each
+  // side. The sides' parts and the ray's own part within the square both come
+  // from these, so that they close whatever the rounding (a line within it of a
+  // side, and parallel, crosses either two sides or none)
+  const float v10 = oc + oa, v01 = oc + ob;
+  const bool s00 = oc >= 0.f, s10 = v10 >= 0.f, s01 = v01 >= 0.f, s11 = v10 + ob >= 0.f;
+  const float ub = __saturatef(-oc * ioa), ut = __saturatef(-v01 * ioa);
+  const float ul = __saturatef(-oc * iob), ur = __saturatef(-v10 * iob);
+  float sum = 0.f;
+  const bool cb = s00 != s10, ct = s01 != s11, cl = s00 != s01, cr = s10 != s11;
+  if (cb || ct || cl || cr) {
+    // ray o between the two crossings
+    const float x1 = cb ? ub : ct ? ut : 0.f, y1 = cb ? 0.f : ct ? 1.f : ul;
+    const float x2 = cr ? 1.f : cl ? 0.f : ut, y2 = cr ? ur : cl ? ul : 1.f;
     const float dx = sgn * ob, dy = -sgn * oa, in = __fdividef(1.0f, fmaf(oa, oa, ob * ob));
-    const float d = fmaf(0.5f, oa + ob, oc) * in, x0 = fmaf(-oa, d, 0.5f), y0 = fmaf(-ob, d, 0.5f);
-    float t0 = fmaf(Ax - x0, dx, (Ay - y0) * dy) * in, t1 = fmaf(Vx - x0, dx, (Vy - y0) * dy) * in;
-    const float ix = __fdividef(1.0f, dx), iy = __fdividef(1.0f, dy);
-    const float xa = -x0 * ix, xb = (1.0f - x0) * ix, ya = -y0 * iy, yb = (1.0f - y0) * iy;
-    t0 = fmaxf(t0, fmaxf(fminf(xa, xb), fminf(ya, yb)));
-    t1 = fminf(t1, fminf(fmaxf(xa, xb), fmaxf(ya, yb)));
-    t1 = fmaxf(t0, t1);
+    const float l = fmaf(x2 - x1, dx, (y2 - y1) * dy) * in;
+    const float x0 = l < 0.f ? x2 : x1, y0 = l < 0.f ? y2 : y1;
+    const float t0 = fmaxf(fmaf(Ax - x0, dx, (Ay - y0) * dy) * in, 0.f);
+    const float t1 = fminf(fmaf(Vx - x0, dx, (Vy - y0) * dy) * in, fabsf(l));
     const float h = fmaf(ha, x0, fmaf(hb, y0, hc)), hs = fmaf(ha, dx, hb * dy);
     const float z = fmaf(za, x0, fmaf(zb, y0, zc)), zs = fmaf(za, dx, zb * dy);
     sum = t1 > t0 ? sgn * stretch((t1 - t0) * hs, fmaf(t0, hs, h), fmaf(t1, hs, h), fmaf(t0, zs, z), fmaf(t1, zs, z)) : 0.f;
   }
   // the square's sides: bottom and top along x, left and right along y
-  const float iha = __fdividef(1.0f, ha), iza = __fdividef(1.0f, za), ioa = __fdividef(1.0f, oa);
-  const float ihb = __fdividef(1.0f, hb), izb = __fdividef(1.0f, zb), iob = __fdividef(1.0f, ob);
 #pragma unroll
   for (int side = 0; side < 4; ++side) {
     const bool along_x = side < 2, far = side & 1;
-    const float hq = along_x ? ha : hb, zq = along_x ? za : zb, oq = along_x ? oa : ob;
+    const float hq = along_x ? ha : hb, zq = along_x ? za : zb;
     const float hp = far ? hc + (along_x ? hb : ha) : hc, zp = far ? zc + (along_x ? zb : za) : zc;
-    const float op = far ? oc + (along_x ? ob : oa) : oc;
-    float lo = 0.f, hi = 1.f;
+    const float u = along_x ? (far ? ut : ub) : (far ? ur : ul);
+    float lo = (along_x ? (far ? s01 : s00) : (far ? s10 : s00)) ? 0.f : u;
+    float hi = (along_x ? (far ? s11 : s10) : (far ? s11 : s01)) ? 1.f : u;
     keep_from(hp, hq, along_x ? iha : ihb, lo, hi);
     keep_from(zp, zq, along_x ? iza : izb, lo, hi);
-    keep_from(op, oq, along_x ? ioa : iob, lo, hi);
     // counter-clockwise: bottom and right forwards, top and left backwards
     const float part = stretch((hi - lo) * hq, fmaf(lo, hq, hp), fmaf(hi, hq, hp), fmaf(lo, zq, zp), fmaf(hi, zq, zp));
     if (hi > lo) sum += (along_x ? !far : far) ? part : -part;
