@@ -34,15 +34,15 @@
 // Hulls thinner than kThinHull pixels and apexes within kThinSector pixels of a
 // hull edge are clipped in FP64 in stage 2: there FP32 rounding of the clip
 // would show next to the pixel's own small value. A pixel's sectors are summed
-// in sixteenths of the accumulator's unit, and the sums added as 64-bit
+// in 64ths of the accumulator's unit, and the sums added as 64-bit
 // fixed-point integers by global atomics, so the image is bitwise reproducible.
 // A last kernel converts them to float.
 //
 // What bounds it: one tetrahedron at a time with a lane per pixel through all
 // of it, lanes took different paths: 8.3 of 32 threads an instruction, 273 ms
 // for 128^3 particles at 1024^2 (1.58e9 pixels of rectangles). Now
-// 56.6 ms: 3 the setup, 11 stage 1, 30 stage 2 (the eight lines and the tests on
-// them, about 800 instructions for 32 pixels), 13 stage 3, at 23 threads an
+// 58 ms: 3 the setup, 11 stage 1, 30 stage 2 (the eight lines and the tests on
+// them, about 800 instructions for 32 pixels), 14 stage 3, at 23 threads an
 // instruction.
 #include "lt_ff.cuh"
 #include "lt_internal.h"
@@ -207,77 +207,89 @@ __device__ __forceinline__ void keep_from(float p, float q, float iq, float& lo,
   if (q == 0.f && p < 0.f) hi = -1.f;
 }
 
-// Six times the integral of h r dh along a stretch on which h goes from h0 to h1,
-// by dh, and r from r0 to r1. (dh from the stretch's length: h1 - h0 would keep
-// the rounding of h far from the hull's edge. The six goes into the divisor at the
-// end: 1/3 and 1/6 in FP32 are both 3e-8 too large, which showed in the frame's
-// mass.)
-__device__ __forceinline__ float stretch(float dh, float h0, float h1, float r0, float r1) {
-  return dh * fmaf(2.0f, fmaf(h0, r0, h1 * r1), fmaf(h0, r1, h1 * r0));
+// Where the line a x + b y + c = 0 crosses the unit square's boundary: its signs
+// at the corners, of which rounding cannot make more than two neighbours differ,
+// and its root on each side. The sides' parts and the line's own part within the
+// square both come from these, so that they close whatever the rounding (a line
+// within it of a side, and parallel, crosses either two sides or none).
+struct Crossing {
+  bool s00, s10, s01, s11;   // >= 0 at (0, 0), (1, 0), (0, 1), (1, 1)
+  float ub, ut, ul, ur;      // roots on the bottom and top (x), left and right (y)
+};
+
+__device__ __forceinline__ Crossing cross_square(float a, float b, float c) {
+  const float ia = __fdividef(1.0f, a), ib = __fdividef(1.0f, b), v10 = c + a, v01 = c + b;
+  return {c >= 0.f, v10 >= 0.f, v01 >= 0.f, v10 + b >= 0.f,
+          __saturatef(-c * ia), __saturatef(-v01 * ia), __saturatef(-c * ib), __saturatef(-v10 * ib)};
+}
+
+// The part of [0, 1] on a side where the line is >= 0, from its signs at the ends
+// and its root.
+__device__ __forceinline__ void keep_side(bool s0, bool s1, float u, float& lo, float& hi) {
+  lo = s0 ? lo : fmaxf(lo, u);
+  hi = s1 ? hi : fminf(hi, u);
+}
+
+// A sector's integral over its part of the unit square is a sixth of the sum,
+// over the stretches of the part's boundary, of w (h0 + h1 + hq): h0 and h1 the
+// hull line's function h at the stretch's ends, hq its value at a point Q, and w
+// the stretch's length times its line's distance from Q, positive where Q lies
+// inside (the divergence theorem for h (p - Q)). This is that term of a ray from
+// the apex (Ax, Ay) to the hull vertex (Vx, Vy), in direction sgn (b, -a).
+__device__ __forceinline__ float ray_term(float a, float b, float c, float sgn, const Crossing& k, float Ax, float Ay,
+                                          float Vx, float Vy, float Qx, float Qy, float ha, float hb, float hc, float hq) {
+  const bool cb = k.s00 != k.s10, ct = k.s01 != k.s11, cl = k.s00 != k.s01, cr = k.s10 != k.s11;
+  // (two crossings or none)
+  const float x1 = cb ? k.ub : ct ? k.ut : 0.f, y1 = cb ? 0.f : ct ? 1.f : k.ul;
+  const float x2 = cr ? 1.f : cl ? 0.f : k.ut, y2 = cr ? k.ur : cl ? k.ul : 1.f;
+  const float dx = sgn * b, dy = -sgn * a, in = __fdividef(1.0f, fmaf(a, a, b * b));
+  const float l = fmaf(x2 - x1, dx, (y2 - y1) * dy) * in;
+  const float x0 = l < 0.f ? x2 : x1, y0 = l < 0.f ? y2 : y1;
+  const float t0 = fmaxf(fmaf(Ax - x0, dx, (Ay - y0) * dy) * in, 0.f);
+  const float t1 = fminf(fmaf(Vx - x0, dx, (Vy - y0) * dy) * in, fabsf(l));
+  const float h = fmaf(ha, x0, fmaf(hb, y0, hc)), hs = fmaf(ha, dx, hb * dy);
+  const float w = fmaf(a, Qx, fmaf(b, Qy, c)) * (t1 - t0);
+  return (cb || ct || cl || cr) && t1 > t0 ? w * (fmaf(t0 + t1, hs, 2.0f * h) + hq) : 0.f;
 }
 
 // Integral of the hull line's function h over the part of the unit square in
-// its sector: h, z, o >= 0, as coefficient triples, z and o the lines of its two
-// rays. (Ax, Ay) and (Vx, Vy): the apex and the vertex on ray o, relative to the
-// square (a far one's rounding does not matter, since the square clips the ray
-// first); sgn: 1 where the vertex lies in direction (ob, -oa) from the apex and
-// the piece's boundary runs there, -1 where both are the other way round.
+// its sector: h, z, o >= 0, as coefficient triples, o the line of the ray from
+// the apex (Ax, Ay) through the vertex (Ox, Oy), z minus that of the ray through
+// (Zx, Zy); all relative to the square.
 //
-// In the coordinates (z, h) the integral is that of h z dh around the piece over
-// the Jacobian J = d(z, h)/d(x, y). The piece's sides on the hull line (h = 0)
-// and on ray z (z = 0) add nothing; left are ray o within the square and the
-// square's four sides within the sector. Every term is of the size of the
-// result, as the functions vanish with the sector's width (an integral along x
-// loses the ratio of the two: 1e-2 of a pixel next to long flat sectors), and all
-// lanes take one path (clipping the square line by line into vertex lists took
-// about 800 instructions at 15 of 32 lanes: 123 ms of a frame against 13).
+// Taken around the part (see ray_term): with Q on the hull line where that cuts
+// the square, its stretch adds nothing; left are the rays' stretches and the
+// square's sides. A term's rounding is that of a vertex's place times h, as for a
+// polygon's, and all lanes take one path (clipping the square line by line into
+// vertex lists took about 800 instructions at 15 of 32 lanes: 123 ms of a frame
+// against 14). An integral in the coordinates (z, h), which needs no second ray,
+// divides by the sine of their angle: 3e-6 of a pixel next to long flat sectors.
 __device__ __forceinline__ float sector_part(float ha, float hb, float hc, float za, float zb, float zc, float oa, float ob,
-                                             float oc, float sgn, float Ax, float Ay, float Vx, float Vy) {
-  // where ray z misses the square, z counts from its smallest value there (a
-  // constant adds nothing around the piece, and would carry its rounding in)
-  zc -= fmaxf(zc + fminf(za, 0.f) + fminf(zb, 0.f), 0.f);
-  const float iha = __fdividef(1.0f, ha), iza = __fdividef(1.0f, za), ioa = __fdividef(1.0f, oa);
-  const float ihb = __fdividef(1.0f, hb), izb = __fdividef(1.0f, zb), iob = __fdividef(1.0f, ob);
-  // where line o crosses the square's sides: its signs at the corners, of which
-  // rounding cannot make more than two neighbours differ, and its root on each
-  // side. The sides' parts and the ray's own part within the square both come
-  // from these, so that they close whatever the rounding (a line within it of a
-  // side, and parallel, crosses either two sides or none)
-  const float v10 = oc + oa, v01 = oc + ob;
-  const bool s00 = oc >= 0.f, s10 = v10 >= 0.f, s01 = v01 >= 0.f, s11 = v10 + ob >= 0.f;
-  const float ub = __saturatef(-oc * ioa), ut = __saturatef(-v01 * ioa);
-  const float ul = __saturatef(-oc * iob), ur = __saturatef(-v10 * iob);
-  float sum = 0.f;
-  const bool cb = s00 != s10, ct = s01 != s11, cl = s00 != s01, cr = s10 != s11;
-  if (cb || ct || cl || cr) {
-    // ray o between the two crossings
-    const float x1 = cb ? ub : ct ? ut : 0.f, y1 = cb ? 0.f : ct ? 1.f : ul;
-    const float x2 = cr ? 1.f : cl ? 0.f : ut, y2 = cr ? ur : cl ? ul : 1.f;
-    const float dx = sgn * ob, dy = -sgn * oa, in = __fdividef(1.0f, fmaf(oa, oa, ob * ob));
-    const float l = fmaf(x2 - x1, dx, (y2 - y1) * dy) * in;
-    const float x0 = l < 0.f ? x2 : x1, y0 = l < 0.f ? y2 : y1;
-    const float t0 = fmaxf(fmaf(Ax - x0, dx, (Ay - y0) * dy) * in, 0.f);
-    const float t1 = fminf(fmaf(Vx - x0, dx, (Vy - y0) * dy) * in, fabsf(l));
-    const float h = fmaf(ha, x0, fmaf(hb, y0, hc)), hs = fmaf(ha, dx, hb * dy);
-    const float z = fmaf(za, x0, fmaf(zb, y0, zc)), zs = fmaf(za, dx, zb * dy);
-    sum = t1 > t0 ? sgn * stretch((t1 - t0) * hs, fmaf(t0, hs, h), fmaf(t1, hs, h), fmaf(t0, zs, z), fmaf(t1, zs, z)) : 0.f;
-  }
-  // the square's sides: bottom and top along x, left and right along y
-#pragma unroll
-  for (int side = 0; side < 4; ++side) {
-    const bool along_x = side < 2, far = side & 1;
-    const float hq = along_x ? ha : hb, zq = along_x ? za : zb;
-    const float hp = far ? hc + (along_x ? hb : ha) : hc, zp = far ? zc + (along_x ? zb : za) : zc;
-    const float u = along_x ? (far ? ut : ub) : (far ? ur : ul);
-    float lo = (along_x ? (far ? s01 : s00) : (far ? s10 : s00)) ? 0.f : u;
-    float hi = (along_x ? (far ? s11 : s10) : (far ? s11 : s01)) ? 1.f : u;
-    keep_from(hp, hq, along_x ? iha : ihb, lo, hi);
-    keep_from(zp, zq, along_x ? iza : izb, lo, hi);
-    // counter-clockwise: bottom and right forwards, top and left backwards
-    const float part = stretch((hi - lo) * hq, fmaf(lo, hq, hp), fmaf(hi, hq, hp), fmaf(lo, zq, zp), fmaf(hi, zq, zp));
-    if (hi > lo) sum += (along_x ? !far : far) ? part : -part;
-  }
-  return __fdividef(sum, 6.0f * fmaf(za, hb, -zb * ha));
+                                             float oc, float Ax, float Ay, float Zx, float Zy, float Ox, float Oy) {
+  const Crossing kz = cross_square(za, zb, zc), ko = cross_square(oa, ob, oc);
+  // Q: the foot of the square's centre on the hull line, or the corner nearest to it
+  const float least = hc + fminf(ha, 0.f) + fminf(hb, 0.f), hq = fmaxf(least, 0.f);
+  const float back = __fdividef(fmaf(0.5f, ha + hb, hc), fmaf(ha, ha, hb * hb));
+  const float Qx = least < 0.f ? fmaf(-ha, back, 0.5f) : ha < 0.f ? 1.f : 0.f;
+  const float Qy = least < 0.f ? fmaf(-hb, back, 0.5f) : hb < 0.f ? 1.f : 0.f;
+  float sum = ray_term(oa, ob, oc, 1.0f, ko, Ax, Ay, Ox, Oy, Qx, Qy, ha, hb, hc, hq) +
+              ray_term(za, zb, zc, -1.0f, kz, Ax, Ay, Zx, Zy, Qx, Qy, ha, hb, hc, hq);
+  const float iha = __fdividef(1.0f, ha), ihb = __fdividef(1.0f, hb);
+  // the square's sides
+  auto side = [&](float p, float q, float iq, bool o0, bool o1, float uo, bool z0, bool z1, float uz, float dist) {
+    float lo = 0.f, hi = 1.f;
+    keep_side(o0, o1, uo, lo, hi);
+    keep_side(z0, z1, uz, lo, hi);
+    keep_from(p, q, iq, lo, hi);
+    if (hi > lo) sum = fmaf(dist * (hi - lo), fmaf(lo + hi, q, 2.0f * p) + hq, sum);
+  };
+  side(hc, ha, iha, ko.s00, ko.s10, ko.ub, kz.s00, kz.s10, kz.ub, Qy);
+  side(hc + hb, ha, iha, ko.s01, ko.s11, ko.ut, kz.s01, kz.s11, kz.ut, 1.0f - Qy);
+  side(hc, hb, ihb, ko.s00, ko.s01, ko.ul, kz.s00, kz.s01, kz.ul, Qx);
+  side(hc + ha, hb, ihb, ko.s10, ko.s11, ko.ur, kz.s10, kz.s11, kz.ur, 1.0f - Qx);
+  // (1 / 6 in two parts: in FP32 alone it is 3e-8 too large, which shows in the
+  // frame's mass)
+  return fmaf(sum, 0.16666667f, sum * -4.967054e-9f);
 }
 
 // Mean column density over pixel (ox, oy) (offsets from the anchor) of one
@@ -654,12 +666,16 @@ struct AreaWarp {
   int2 near[64];             // pixels that stage 1 kept: slot, index in the rectangle
   float line[8][32];         // stage 2's lines at the pixel's corner: four of the hull, four rays
   int slot[32];              // stage 2's tetrahedra
-  unsigned sum[2][32];       // stage 2's pixels: sectors clipped in stage 3, in sixteenths of a unit
+  unsigned sum[2][32];       // stage 2's pixels: sectors clipped in stage 3, in 64ths of a unit
   unsigned char job[128];    // pixels of stage 2 << 2 | sector
 };
 
 // Sums past this many units go to the image by themselves.
 constexpr float kDirect = 1.0e12f;
+// A pixel's sectors are summed in 64ths of a unit: rounded to a unit only once
+// (16ths: 0.8% more rounding where a thousand tetrahedra meet in a pixel).
+constexpr int kPartBits = 6;
+constexpr float kParts = 64.0f;
 
 __global__ void __launch_bounds__(kAreaThreads, 4) k_area(AreaArgs a) {
   extern __shared__ __align__(16) float area_smem[];
@@ -772,22 +788,19 @@ __global__ void __launch_bounds__(kAreaThreads, 4) k_area(AreaArgs a) {
         const float ha = t.hull_h[0][e], hb = t.hull_h[1][e];
         const float ra = t.ray_h[0][e], rb = t.ray_h[1][e], rc = S.line[4 + e][o];
         const float ga = -t.ray_h[0][f], gb = -t.ray_h[1][f], gc = -S.line[4 + f][o];
-        // z: the ray at the larger angle to the hull line
-        const bool first_ray = fabsf(fmaf(ra, hb, -rb * ha)) >= fabsf(fmaf(ga, hb, -gb * ha));
-        const int w = first_ray ? f : e;
-        const float in = sector_part(ha, hb, S.line[e][o], first_ray ? ra : ga, first_ray ? rb : gb, first_ray ? rc : gc,
-                                     first_ray ? ga : ra, first_ray ? gb : rb, first_ray ? gc : rc, first_ray ? -1.0f : 1.0f,
-                                     t.qx - ox, t.qy - oy, (t.vx_h[w] - ox) + t.vx_l[w], (t.vy_h[w] - oy) + t.vy_l[w]);
+        const float in = sector_part(ha, hb, S.line[e][o], ga, gb, gc, ra, rb, rc, t.qx - ox, t.qy - oy,
+                                     (t.vx_h[f] - ox) + t.vx_l[f], (t.vy_h[f] - oy) + t.vy_l[f],
+                                     (t.vx_h[e] - ox) + t.vx_l[e], (t.vy_h[e] - oy) + t.vy_l[e]);
         const float v = t.k[e] * in;
-        if (v < 1.3e8f) {
+        if (v < 3.3e7f) {
           // (rounding can leave a part next to nothing on either side of zero:
           // signed, so that the parts' errors do not add up)
-          const int i = __float2int_rn(16.0f * fmaxf(v, -1.3e8f));
+          const int i = __float2int_rn(kParts * fmaxf(v, -3.3e7f));
           const unsigned u = (unsigned)i;
           const unsigned hi = (i < 0 ? ~0u : 0u) + (atomicAdd(&S.sum[0][o], u) > ~u ? 1u : 0u);
           if (hi) atomicAdd(&S.sum[1][o], hi);
         } else if (v < kDirect) {
-          const unsigned long long u = __float2ull_rn(16.0f * v);
+          const unsigned long long u = __float2ull_rn(kParts * v);
           const unsigned lo = (unsigned)u;
           const unsigned hi = (unsigned)(u >> 32) + (atomicAdd(&S.sum[0][o], lo) > ~lo ? 1u : 0u);
           if (hi) atomicAdd(&S.sum[1][o], hi);
@@ -800,10 +813,10 @@ __global__ void __launch_bounds__(kAreaThreads, 4) k_area(AreaArgs a) {
     if (lane < n) {
       if (whole < kDirect) {
         unsigned long long u = (unsigned long long)max((long long)((unsigned long long)S.sum[1][lane] << 32 | S.sum[0][lane]), 0LL);
-        u += whole < 2.6e8f ? (unsigned long long)__float2uint_rn(16.0f * whole) : __float2ull_rn(16.0f * whole);
-        area_add_units(a, F, px, py, (u + 7ull + ((u >> 4) & 1ull)) >> 4);  // (to the nearest, halves to even)
+        u += whole < 6.6e7f ? (unsigned long long)__float2uint_rn(kParts * whole) : __float2ull_rn(kParts * whole);
+        area_add_units(a, F, px, py, (u + 31ull + ((u >> kPartBits) & 1ull)) >> kPartBits);  // (to the nearest, halves to even)
       } else {
-        area_add_units(a, F, px, py, (unsigned long long)max((long long)((unsigned long long)S.sum[1][lane] << 32 | S.sum[0][lane]), 0LL) >> 4);
+        area_add_units(a, F, px, py, (unsigned long long)max((long long)((unsigned long long)S.sum[1][lane] << 32 | S.sum[0][lane]), 0LL) >> kPartBits);
         area_add(a, F, px, py, whole);
       }
     }
