@@ -417,79 +417,88 @@ __device__ __noinline__ bool setup_f64(const AreaArgs& a, const FrameDev& F, int
   if (!ok || tf.V == 0.0) return false;
   const double hl = (double)a.L.box / a.L.N;
   const double base[3] = {i * hl, j * hl, k * hl};
-  double P[4][2];
+  double P[4][2], eps[2] = {0.0, 0.0};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     double w[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) w[q] = base[q] + tf.v[c][q];
-    P[c][0] = (F.rd[0] * w[0] + F.rd[1] * w[1] + F.rd[2] * w[2] - F.lod[0]) / F.pxd[0];
-    P[c][1] = (F.ud[0] * w[0] + F.ud[1] * w[1] + F.ud[2] * w[2] - F.lod[1]) / F.pxd[1];
-  }
-  // the apex and the hull, counter-clockwise: a vertex inside the triangle of
-  // the other three is the apex
-  double Ax = 0.0, Ay = 0.0, Hx[4], Hy[4];
-  int n = 0;
-  int inner = -1;
-  for (int c = 0; c < 4 && inner < 0; ++c) {
-    const int p = (c + 1) & 3, q = (c + 2) & 3, r = (c + 3) & 3;
-    const double o = orient(P[p][0], P[p][1], P[q][0], P[q][1], P[r][0], P[r][1]);
-    if (o == 0.0) continue;
-    const double s1 = orient(P[p][0], P[p][1], P[q][0], P[q][1], P[c][0], P[c][1]) * o;
-    const double s2 = orient(P[q][0], P[q][1], P[r][0], P[r][1], P[c][0], P[c][1]) * o;
-    const double s3 = orient(P[r][0], P[r][1], P[p][0], P[p][1], P[c][0], P[c][1]) * o;
-    // on the boundary counts too: coincident projections (the undeformed
-    // lattice seen along an axis) put the apex on a hull vertex or edge,
-    // where the triangles beside it have no area
-    if (s1 >= 0.0 && s2 >= 0.0 && s3 >= 0.0) {
-      inner = c;
-      Ax = P[c][0];
-      Ay = P[c][1];
-      const bool ccw = o > 0.0;
-      const int ord[3] = {p, ccw ? q : r, ccw ? r : q};
-      for (int e = 0; e < 3; ++e) {
-        Hx[e] = P[ord[e]][0];
-        Hy[e] = P[ord[e]][1];
-      }
-      n = 3;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double* axis = q == 0 ? F.rd : F.ud;
+      P[c][q] = (axis[0] * w[0] + axis[1] * w[1] + axis[2] * w[2] - F.lod[q]) / F.pxd[q];
+      // its rounding: a few 2^-53 of the terms
+      const double size = fabs(axis[0] * w[0]) + fabs(axis[1] * w[1]) + fabs(axis[2] * w[2]) + fabs(F.lod[q]);
+      eps[q] = fmax(eps[q], 0x1p-50 * size / F.pxd[q]);
     }
   }
-  if (inner < 0) {
-    // four vertices in convex position: vertex 0's diagonal partner d is the
-    // one whose segment from vertex 0 separates the other two
-    int d = -1, u = -1, w = -1;
-    for (int c = 1; c < 4 && d < 0; ++c) {
-      const int p = c == 1 ? 2 : 1, q = 6 - c - p;
-      const double sp = orient(P[0][0], P[0][1], P[c][0], P[c][1], P[p][0], P[p][1]);
-      const double sq = orient(P[0][0], P[0][1], P[c][0], P[c][1], P[q][0], P[q][1]);
-      if ((sp > 0.0 && sq < 0.0) || (sp < 0.0 && sq > 0.0)) {
-        d = c;
-        // counter-clockwise: 0, u, d, w with u on the right of 0 -> d
-        u = sp < 0.0 ? p : q;
-        w = sp < 0.0 ? q : p;
-      }
+  // the apex and the hull, counter-clockwise, by the signed areas c_i = (-1)^i
+  // orient(the others), which sum to zero: a lone sign marks the vertex inside the
+  // triangle of the others, two of each the diagonals. An area of rounding's size
+  // counts as none: the vertex of the lone sign then lies on a hull edge, or, with
+  // two such areas, on a hull vertex (lattices seen along an axis at which they
+  // are at rest), and the triangles beside it have no area.
+  double D[3][2], dmax[2] = {0.0, 0.0};
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      D[c][q] = P[c + 1][q] - P[0][q];
+      dmax[q] = fmax(dmax[q], fabs(D[c][q]));
     }
-    if (d < 0) return false;
-    const double o0 = orient(P[u][0], P[u][1], P[w][0], P[w][1], P[0][0], P[0][1]);
-    const double od = orient(P[u][0], P[u][1], P[w][0], P[w][1], P[d][0], P[d][1]);
-    if (!((o0 > 0.0 && od < 0.0) || (o0 < 0.0 && od > 0.0))) return false;  // not a crossing
-    const double tt = o0 / (o0 - od);
+  const double o12 = D[0][0] * D[1][1] - D[0][1] * D[1][0], o13 = D[0][0] * D[2][1] - D[0][1] * D[2][0];
+  const double o23 = D[1][0] * D[2][1] - D[1][1] * D[2][0];
+  const double cc[4] = {(o12 + o23) - o13, -o23, o13, -o12};
+  double none = 8.0 * (eps[0] * dmax[1] + eps[1] * dmax[0]);
+  int pos = 0, neg = 0;
+  for (int c = 0; c < 4; ++c) {
+    if (cc[c] > none) pos |= 1 << c;
+    if (cc[c] < -none) neg |= 1 << c;
+  }
+  if (pos == 0 || neg == 0) {  // a whole hull of that size: by the signs as they are
+    none = 0.0;
+    pos = neg = 0;
+    for (int c = 0; c < 4; ++c) {
+      if (cc[c] > 0.0) pos |= 1 << c;
+      if (cc[c] < 0.0) neg |= 1 << c;
+    }
+    if (pos == 0 || neg == 0) return false;
+  }
+  double Ax, Ay, Hx[4], Hy[4];
+  int n, ord[4];
+  if (__popc(pos) == 2 && __popc(neg) == 2) {
+    // the diagonals are (0, d) and (u, w), vertex 0 and d as far from the other as
+    // their triangles' areas
+    const int same = pos & 1 ? pos : neg;
+    const int d = (same >> 1) & 1 ? 1 : (same >> 2) & 1 ? 2 : 3;
+    int u = d == 1 ? 2 : 1, w = 6 - d - u;
+    if (orient(P[u][0], P[u][1], P[w][0], P[w][1], P[0][0], P[0][1]) < 0.0) { const int x = u; u = w; w = x; }
+    const double tt = cc[d] / (cc[d] + cc[0]);
     Ax = P[0][0] + tt * (P[d][0] - P[0][0]);
     Ay = P[0][1] + tt * (P[d][1] - P[0][1]);
-    const int ord[4] = {0, u, d, w};
-    for (int e = 0; e < 4; ++e) {
-      Hx[e] = P[ord[e]][0];
-      Hy[e] = P[ord[e]][1];
-    }
+    ord[0] = 0; ord[1] = u; ord[2] = d; ord[3] = w;
     n = 4;
+  } else {
+    const int c = 31 - __clz(__popc(pos) == 1 ? pos : neg);
+    const int p = (c + 1) & 3, q = (c + 2) & 3, r = (c + 3) & 3;
+    const bool ccw = orient(P[p][0], P[p][1], P[q][0], P[q][1], P[r][0], P[r][1]) > 0.0;
+    Ax = P[c][0];
+    Ay = P[c][1];
+    ord[0] = p; ord[1] = ccw ? q : r; ord[2] = ccw ? r : q; ord[3] = p;
+    n = 3;
   }
-  double area2 = 0.0, emax = 0.0;
+  for (int e = 0; e < 4; ++e) {
+    Hx[e] = P[ord[e]][0];
+    Hy[e] = P[ord[e]][1];
+  }
+  // twice the hull's area: the two triangles beside a diagonal, or the one around
+  // the apex
+  const double area2 = 0.5 * (fabs(cc[0]) + fabs(cc[1]) + fabs(cc[2]) + fabs(cc[3]));
+  double emax = 0.0;
   for (int e = 0; e < n; ++e) {
     const int f = e + 1 == n ? 0 : e + 1;
-    area2 += Hx[e] * Hy[f] - Hx[f] * Hy[e];
     emax = fmax(emax, hypot(Hx[f] - Hx[e], Hy[f] - Hy[e]));
   }
-  if (!(area2 > 0.0)) return false;
   // column density at the apex: 3 m / (hull area in world units)
   const double h = 3.0 * a.m_tet / (0.5 * area2 * F.pxd[0] * F.pxd[1]);
   t.ax = (int)fmin(fmax(floor(Ax), -1.0e9), 1.0e9);
@@ -506,7 +515,9 @@ __device__ __noinline__ bool setup_f64(const AreaArgs& a, const FrameDev& F, int
     const float2 vx = split_ff(Hx[e] - t.ax), vy = split_ff(Hy[e] - t.ay);
     t.vx_h[e] = vx.x; t.vx_l[e] = vx.y;
     t.vy_h[e] = vy.x; t.vy_l[e] = vy.y;
-    const double dA = line_f64(t.hull_h, t.hull_l, e, qx, qy);
+    const double len = fabs(Hx[f] - Hx[e]) + fabs(Hy[f] - Hy[e]);
+    double dA = line_f64(t.hull_h, t.hull_l, e, qx, qy);
+    if (dA * len <= none) dA = 0.0;  // twice the area of the apex's triangle
     t.k[e] = dA > 0.0 ? (float)(h / dA * a.inv_unit) : 0.0f;
     // an apex next to a hull edge: a long thin face whose FP32 clip would lose
     // its relative accuracy while k_e grows as 1 / dA

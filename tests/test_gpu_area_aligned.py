@@ -87,3 +87,18 @@ def test_lattice_planes_beside_pixel_edges(R, N, sign, shift):
     # (a window that begins before the box loses `shift` of its first row and column)
     assert np.all(np.abs(got - 1.0) <= 1e-5)
     assert abs(got.mean() - 1.0) <= 1e-6
+
+
+@pytest.mark.parametrize("N,W,H,kind", [(5, 20, 15, "still x"), (7, 21, 35, "still x"), (9, 36, 45, "still y"),
+                                        (11, 22, 33, "still x"), (13, 52, 39, "still y"), (20, 60, 60, "still x")])
+def test_projections_that_nearly_coincide(R, N, W, H, kind):
+    """FP16 lattices with an axis at rest: vertices of a tetrahedron that project
+    onto one line, or onto one point, but for the rounding of their FP64
+    coordinates (box / N is not a power of two)."""
+    p, x = particles(N, kind, True)
+    R.build_tets(torch.from_numpy(p).cuda(), N)
+    got = R.render_area(ortho_z(W, H)).cpu().numpy().astype(np.float64)
+    R.sync()
+    ref = oracle.render_area(x, N, ortho_z(W, H))
+    assert np.all(np.abs(got - ref) <= 1e-5 * np.maximum(ref, 1.0))
+    assert abs(got.mean() - 1.0) <= 1e-6
