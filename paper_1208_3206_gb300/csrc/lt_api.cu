@@ -67,7 +67,7 @@ struct lt_ctx {
   size_t frag_cap = 0;
   unsigned long long* h_u64 = nullptr;  // pinned scratch
   cudaEvent_t sized = nullptr;          // the lists' size has reached h_u64
-  // zero-volume tetrahedra: one bit per tetrahedron, a byte per (snapshot, cube)
+  // a byte per (snapshot, cube): zero-volume tetrahedra, a bit each, and whether a corner is not finite
   unsigned char* d_degen = nullptr;
   size_t degen_cap = 0;
   // resampling: fixed-point cells

@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(kBackThreads, 4) k_backward(Lattice L, const F
   const int s = threadIdx.x / kBackCubes, c = threadIdx.x % kBackCubes;
   for (long long base = (long long)blockIdx.x * kBackCubes; base < ncube; base += (long long)gridDim.x * kBackCubes) {
     const long long cube = base + c;
-    const bool drawn = cube < ncube && !tet_degenerate(L, snap, cube, s);  // zero volume: contributes nothing
+    // zero volume, or a cube with a corner that is not finite: contributes nothing
+    const bool drawn = cube < ncube && !(cube_mask(L, snap, cube) & (1u << s | kNonFiniteCube));
     float G[2][3];  // corner items threadIdx.x and, for the first threads, kBackThreads further
 #pragma unroll
     for (int h = 0; h < 2; ++h) G[h][0] = G[h][1] = G[h][2] = 0.f;

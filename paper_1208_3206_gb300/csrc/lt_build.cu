@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_build_tets(BuildArgs a) {
       }
     }
     __syncwarp();
-    if (cube < ncube) a.degen[soff + cube] = (unsigned char)wzero[lane];
+    if (cube < ncube) a.degen[soff + cube] = (unsigned char)(wzero[lane] | (finite ? 0u : kNonFiniteCube));
     if (a.rho_out) {
       const long long w0 = base + wbase;  // the warp's first cube
       float* out = a.rho_out + (soff + w0) * 6;

@@ -121,6 +121,12 @@ __device__ __forceinline__ unsigned div_n(const Lattice& L, unsigned n) {
 #endif
 
 // True when tetrahedron s of `cube` in snapshot `snap` has zero volume.
+// The cube's byte: a bit for each tetrahedron of zero volume, and kNonFiniteCube
+// where a corner is not finite (the projections draw nothing of such a cube).
+constexpr unsigned kNonFiniteCube = 64u;
+__device__ __forceinline__ unsigned cube_mask(const Lattice& L, int snap, long long cube) {
+  return L.degen ? (unsigned)__ldg(L.degen + (long long)snap * L.n_particles + cube) : 0u;
+}
 __device__ __forceinline__ bool tet_degenerate(const Lattice& L, int snap, long long cube, int s) {
   return L.degen && ((__ldg(L.degen + (long long)snap * L.n_particles + cube) >> s) & 1u);
 }
