@@ -317,7 +317,10 @@ __global__ void __launch_bounds__(kResampleThreads) k_resample(ResampleArgs a) {
   if (tau < ntet) {
     const long long cube = tau / 6;
     const int s = (int)(tau - 6 * cube);
-    if (!tet_degenerate(a.L, a.snapshot, cube, s)) {  // zero volume: contributes nothing
+    const unsigned mask = cube_mask(a.L, a.snapshot, cube);
+    if (mask & kNonFiniteCube) {
+      atomicOr(&a.ctr->errors, kErrNonFinite);
+    } else if (!((mask >> s) & 1u)) {  // zero volume: contributes nothing
       int i, j, k;
       cube_ijk(a.L, cube, i, j, k);
       have = a.use_ff ? resample_fixed(a, i, j, k, s, S.tets[lane]) : 2;

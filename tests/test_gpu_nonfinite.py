@@ -65,3 +65,14 @@ def test_gradient_of_bad_cubes(R, half, value):
     assert torch.equal(grads[0][far], grads[1][far])
     assert bool(torch.isfinite(grads[1]).all())
     assert float(grads[1][31].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("weight", ["density", "streams"])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("half", [False, True])
+def test_grid_of_bad_cubes(R, half, value, weight):
+    _, pos = bad_lattice(R, 2, 3, value, half)
+    R.build_tets(pos, 2)
+    assert latched(R)
+    assert float(R.resample(12, weight=weight).abs().max()) == 0.0
+    assert latched(R)
