@@ -49,6 +49,7 @@ namespace lt {
 constexpr int kResampleThreads = 64;
 constexpr int kZBits = 42;  // fraction bits of a height in cells
 constexpr long long kZOne = 1LL << kZBits;
+constexpr float kTieAxis = 0.3719f;  // see the vertical faces of resample_fixed
 
 struct ResampleArgs {
   Lattice L;
@@ -116,7 +117,8 @@ __device__ __noinline__ bool resample_f64(const ResampleArgs& a, int i, int j, i
     r.d.nx[f] = t.n[f][0];
     r.d.ny[f] = t.n[f][1];
     r.d.d[f] = t.d[f];
-    r.d.inz[f] = t.n[f][2] != 0.0 ? 1.0 / t.n[f][2] : 0.0;
+    const double big = fmax(fabs(t.n[f][0]), fabs(t.n[f][1]));
+    r.d.inz[f] = fabs(t.n[f][2]) > 1e-12 * big ? 1.0 / t.n[f][2] : 0.0;
   }
   r.d.q = a.weight == 0 ? a.m_tet / fabs(t.V) : 1.0;
   r.d.qx = i * h;
@@ -135,6 +137,13 @@ __device__ __noinline__ bool resample_f64(const ResampleArgs& a, int i, int j, i
   r.B0 = (int)B0;
   r.wa = (int)(A1 - A0) + 1;
   r.wb = (int)(B1 - B0) + 1;
+  // columns on a vertical face: on one side of it, as in the integer form
+  const double tie = (8.0 * ((double)r.wa + (double)r.wb + 8.0)) / (double)kZOne * a.gs;
+  for (int f = 0; f < 4; ++f)
+    if (r.d.inz[f] == 0.0) {
+      const double nx = r.d.nx[f], ny = r.d.ny[f];
+      r.d.d[f] += (nx + (double)kTieAxis * ny < 0.0 ? tie : -tie) * fmax(fabs(nx), fabs(ny));
+    }
   r.form = 2;
   return true;
 }
@@ -192,6 +201,8 @@ __device__ __forceinline__ int resample_fixed(const ResampleArgs& a, int i, int 
     m[3][q] = e[0][u] * e[1][t] - e[0][t] * e[1][u];
     m[0][q] = -((m[1][q] + m[2][q]) + m[3][q]);
   }
+  // (face 0 is vertical where its sum is the rounding of its terms)
+  if (fabsf(m[0][2].h) <= 0x1p-38f * (fabsf(m[1][2].h) + fabsf(m[2][2].h) + fabsf(m[3][2].h))) m[0][2] = {0.f, 0.f};
   // face f holds vertex 0 (f = 1..3) or vertex 1 (f = 0); inside m . (p - v) / det >= 0
   int upper = 0, vertical = 0;
 #pragma unroll
@@ -223,6 +234,15 @@ __device__ __forceinline__ int resample_fixed(const ResampleArgs& a, int i, int 
     r.f.A[f] = to_fixed(A);
     r.f.B[f] = to_fixed(B);
     r.f.C[f] = to_fixed(C);
+    if ((vertical >> f) & 1) {
+      // a column on the face, within rounding, belongs to the tetrahedron on the
+      // one side and not to that on the other (a lattice at rest has whole planes
+      // of columns on faces: counted on both sides they held up to four times
+      // their mass). The side: by the direction's sign along an axis that no
+      // lattice face is parallel to, so that a component's rounding does not matter
+      const long long tie = 8LL * (w[0] + w[1] + 8);
+      r.f.C[f] += A.h + kTieAxis * B.h > 0.f ? tie : -tie - 1;
+    }
   }
   r.f.upper = upper;
   r.f.vertical = vertical;
