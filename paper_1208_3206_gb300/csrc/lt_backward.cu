@@ -78,7 +78,7 @@ __device__ __forceinline__ void backward_tet(const Lattice& L, const FrameDev& F
     return;
   float ia[4];  // (the spans have room for its rounding)
 #pragma unroll
-  for (int e = 0; e < 4; ++e) ia[e] = fast_rcp(t.a[e]);
+  for (int e = 0; e < 4; ++e) ia[e] = inv_or_zero(t.a[e]);
   int sx0, sx1, sy0, sy1;
   const float axa = P.axh + P.axl, aya = P.ayh + P.ayl;
   shift_range(axa + t.xmin, axa + t.xmax, -0.5f, (float)F.W - 0.5f, (float)F.W, F.wrap != 0, sx0, sx1);

@@ -479,6 +479,14 @@ __device__ __forceinline__ float diff2(float a, float b, float c, float d) {
 template <bool PIN = false>
 __device__ __forceinline__ float cross2(float ax, float ay, float bx, float by) { return diff2<PIN>(ax, by, ay, bx); }
 
+// 1 / a to an ulp, or 0 for a == 0 (an edge function constant along the row).
+// (__fdividef returns 0 from 2^126 on, which a steep sliver's |a| can pass.)
+__device__ __forceinline__ float inv_or_zero(float a) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return a != 0.0f ? r : 0.0f;
+}
+
 // Conditionally swap two scalars.
 __device__ __forceinline__ void cswap(bool s, float& p, float& q) {
   const float tp = p, tq = q;

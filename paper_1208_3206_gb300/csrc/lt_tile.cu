@@ -83,14 +83,6 @@ __device__ __forceinline__ unsigned long long pack_frag(unsigned tau, int sx, in
          ((unsigned long long)(unsigned)Y << 52);
 }
 
-// 1 / a to an ulp, or 0 for a == 0 (an edge function constant along the row).
-// (__fdividef returns 0 from 2^126 on, which a steep sliver's |a| can pass.)
-__device__ __forceinline__ float inv_or_zero(float a) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return a != 0.0f ? r : 0.0f;
-}
-
 // Narrow [lo, hi] to the X where a X + rr >= 0 (rr the row term b Y + c). An
 // edge constant along the row (a == 0) does not constrain it: where its rr is
 // negative the walk's values are too, and add nothing.
