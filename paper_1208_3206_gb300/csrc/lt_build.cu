@@ -200,12 +200,15 @@ __global__ void __launch_bounds__(kBuildThreads) k_build_tets(BuildArgs a) {
         if (a.rho_out) {
           float rho = 0.0f;
           if (finite && V != 0.0f) {
+            const float v = fabsf(V);
             if (a.use_ff) {
-              // m / |V| to about 2^-44 before its one rounding
-              const float v = fabsf(V), rv = __frcp_rn(v), q = __fmul_rn(a.m_ff.h, rv);
-              rho = __fadd_rn(q, __fmul_rn(__fadd_rn(__fmaf_rn(-q, v, a.m_ff.h), a.m_ff.l), rv));
+              // m / |V| to about 2^-44 before its one rounding (the residual of a volume
+              // past FP32's range, of particles far outside the box, is taken at the
+              // range's end: 0 times infinity is no number)
+              const float rv = __frcp_rn(v), q = __fmul_rn(a.m_ff.h, rv);
+              rho = __fadd_rn(q, __fmul_rn(__fadd_rn(__fmaf_rn(-q, fminf(v, 3.4028235e38f), a.m_ff.h), a.m_ff.l), rv));
             } else {
-              rho = (float)(a.m / (double)fabsf(V));
+              rho = (float)(a.m / (double)v);
             }
           }
           wrho[lane * 6 + s] = rho;
