@@ -115,7 +115,7 @@ typedef struct {
   long long entries;         /* (tile, cube) bin entries of the last lt_project_bin */
   long long capacity;        /* reserved bin entries */
   long long degenerate;      /* tetrahedra with V == 0 found by lt_build_tets */
-  long long fp64_fallbacks;  /* volumes recomputed in FP64 by lt_build_tets */
+  long long fp64_fallbacks;  /* volumes recomputed by lt_build_tets beyond FP32 (float-float, or FP64 where that cancels) */
   long long inverted;        /* tetrahedra with V > 0 (orientation flipped vs t = 0) */
   long long nonfinite;       /* non-finite positions seen */
   long long behind_eye;      /* cubes skipped because they straddle a perspective eye plane */
@@ -154,9 +154,10 @@ lt_status lt_get_config(const lt_ctx* ctx, lt_config* out);
  * owned, read by every later call) for a lattice of N^3 particles in a
  * periodic box of edge `box` holding `total_mass`. Checks every position
  * for finiteness and computes, for every tetrahedron of every snapshot, the
- * signed volume V (FP32 from displacement differences, recomputed in FP64
- * when |V| < 0.1 of a lattice cell, where the FP32 error bound would pass
- * 1e-5; this covers every near-degenerate sheet tetrahedron at caustics) and
+ * signed volume V (FP32 from displacement differences, recomputed from exact
+ * edges in float-float, or in FP64 where that cancels by more than 2^18, when
+ * |V| < 0.1 of a lattice cell, where the FP32 error bound would pass 1e-5;
+ * this covers every near-degenerate sheet tetrahedron at caustics) and
  * rho = m / |V| (0 when V == 0). Tetrahedra with V == 0 are marked in a
  * context-owned mask (one byte per cube and snapshot) and contribute nothing
  * to any later render. If d_rho is not NULL it receives rho as float
@@ -193,9 +194,10 @@ lt_status lt_project_bin(lt_ctx* ctx, const lt_camera* cams, int n_frames, const
  * into on-chip fixed-point integer sums (so the image is bit-reproducible
  * whatever the order), and stores every pixel once. Fragments whose FP32
  * value may be off by more than 1e-5 of max(value, mean column density)
- * (thin slivers, steep edges) are re-evaluated exactly in FP64 by clipping
- * the pixel ray against the four faces; tetrahedra with V == 0 contribute
- * nothing. A graph replay whose lists outgrew their capacity draws only the
+ * (thin slivers, steep edges) are re-evaluated in FP64 from the stored
+ * positions: by the pyramid about the pixel ray, or for a tetrahedron within
+ * 2e-5 of flat by clipping the ray against its four faces; tetrahedra with
+ * V == 0 contribute nothing. A graph replay whose lists outgrew their capacity draws only the
  * entries the lists hold and latches LT_ERR_CAPACITY.
  * d_image: float [n_frames][H][W] (caller owned). d_mass (may be NULL):
  * double [n_frames], per frame the sum of pixel values times the pixel area
@@ -245,9 +247,12 @@ lt_status lt_render_backward(lt_ctx* ctx, const float* d_dL_dimage, float* d_dL_
  * (Eq. 3), so a cell holds rho dl, its mass over its face area;
  * LT_WEIGHT_STREAMS: q_t = 1, so a cell over g is the mean number of streams
  * on its line. Each (tetrahedron, line) interval is found by clipping the
- * line against the four face planes, to about 2^-40 of a cell; the cells are summed as
- * 64-bit fixed-point integers (2^-frac_bits of the mean cell), so the grid
- * is bitwise reproducible. Tetrahedra with V == 0 contribute nothing.
+ * line against the four face planes, whose heights are good to 2^-43 of a cell
+ * for every column that the tetrahedron spans (2^-40 for eight, 2^-32 for two
+ * thousand). A line on a vertical face belongs to one side of it. The cells are
+ * summed as 64-bit fixed-point integers (2^-frac_bits of the mean cell), so the
+ * grid is bitwise reproducible. Tetrahedra with V == 0, and cubes with a corner
+ * that is not finite, contribute nothing.
  * Asynchronous, without bins of its own; render or count afterwards only after
  * a new lt_project_bin (LT_ERR_STATE). Keeps an n^3 array of 64-bit cells in
  * the context.
@@ -266,8 +271,9 @@ lt_status lt_resample(lt_ctx* ctx, int n, int weight, int snapshot, float* d_gri
  * ((a + 1/2) box / n, (b + 1/2) box / n, z0), the sum over the tetrahedra
  * that contain it (every periodic copy counts) of rho_t = m / |V_t|
  * (LT_WEIGHT_DENSITY: the total density) or of 1 (LT_WEIGHT_STREAMS: the
- * number of streams). The containment test is done in FP64 against the four
- * face planes; a point on a face counts for both tetrahedra sharing it.
+ * number of streams). Containment is decided as FP64 decides it against the
+ * four face planes (in FP32 where its rounding cannot matter); a point on a
+ * face counts for both tetrahedra sharing it.
  * Sums are 64-bit fixed point in units of 2^-frac_bits of the mean density
  * (of one stream: counts are exact), so the slice is bitwise reproducible.
  * Tetrahedra with V == 0 contribute nothing. Asynchronous; leaves the bins

@@ -1,9 +1,10 @@
 // lt_bin.cu -- project-and-bin pass: for every (frame, cube) the screen
 // tiles overlapped by the cube's projected bounding box; warp-aggregated
 // per-tile counts (the count pass also keeps each cube's tile rectangle, so
-// the scatter does not project again), a device exclusive scan, a scatter of
-// cube ids into per-tile lists, and the (frame, tile) work list ordered by
-// descending list length (bucketed by log2 of the length).
+// the scatter does not project again), a device exclusive scan (which also
+// writes the total and clears the scatter's cursors), a scatter of cube ids
+// into per-tile lists, and the work list: every (frame, tile) list in chunks,
+// ordered by descending length (bucketed by log2 of the length).
 #include "lt_internal.h"
 
 namespace lt {

@@ -28,10 +28,12 @@
 //     atomic. Integer sums do not depend on the order of the adds, so the grid is
 //     bitwise reproducible. Consecutive warps take consecutive cubes, whose cells
 //     share the L2.
-// A tetrahedron whose volume cancels beyond float-float, or with a face so near
-// to vertical (2^12 cells per column) or a number so large that the integers
-// would not hold it to about 2^-40 of a cell, is clipped in FP64. A last kernel
-// converts the integer grid to float.
+// A and B are rounded to 2^-43 of a cell, so a height is good to that times the
+// columns that the tetrahedron spans: 2^-40 for eight of them, 2^-32 for two
+// thousand (a cell holds FP32 numbers). A tetrahedron whose volume cancels beyond
+// float-float, with a face so near to vertical (2^12 cells per column) or numbers
+// so large that the integers would not hold them, is clipped in FP64. A last
+// kernel converts the integer grid to float.
 //
 // What bounds it: with the planes, the intervals and their pieces in FP64 the
 // FP64 pipe took 148 ms for 128^3 particles onto 512^3 cells (1.6e8 intervals,

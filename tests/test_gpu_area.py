@@ -1,8 +1,9 @@
 """GPU parity of the area-averaged pixels (lt_render_area) against the FP64
 oracle (oracle.render_area) on the same seeded inputs: every pixel within
 1e-4 of max(pixel, mean column density), the frame mass within 1e-6.
-The GPU sets up each tetrahedron's pyramid in FP64 and evaluates each line
-at the pixel's corner in float-float; the clip runs in FP32 (FP64 for hulls
+The GPU sets up each tetrahedron's pyramid in float-float (FP64 for
+projections near to degenerate) and evaluates each line at the pixel's corner
+in float-float; the integral over the pixel runs in FP32 (FP64 for hulls
 thinner than 1/20 pixel), so its error is a few 1e-7 of the largest column
 density in the pixel plus the 64-bit fixed-point rounding."""
 import numpy as np
