@@ -59,6 +59,17 @@ def test_values_of_a_tile_size(Renderer, tile):
         assert abs(img[y, x] - float.fromhex(v)) <= 2.0 ** -23 * float.fromhex(v), (y, x)
 
 
+def test_values_in_perspective(Renderer):
+    """The same in perspective at 64-pixel tiles, where the pixels moved by 7e-6
+    to 1.1e-5; approximate reciprocals in the projection leave 2e-6."""
+    R = Renderer(tile=64)
+    R.build_tets(sheets(24, 2), 24)
+    R.project_bin(dict(type="persp", W=300, H=280, eye=(0.5, -1.4, 0.9), fwd=(0.0, 1.0, -0.21), up=(0, 0, 1), fov_y_deg=50.0))
+    img = R.render_tiles().cpu().numpy().reshape(280, 300).astype(np.float64)
+    for (y, x), v in {(191, 128): 1.7096133, (191, 66): 1.8924608, (105, 190): 1.1309264}.items():
+        assert abs(img[y, x] - v) <= 2e-6 * v, (y, x)
+
+
 @pytest.mark.parametrize("W,H", [(300, 280), (1040, 1024)])
 def test_tile_left_open(Renderer, W, H):
     """The default tile is 16 pixels whatever the frame's size, and writing back
