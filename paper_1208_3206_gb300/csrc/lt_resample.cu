@@ -115,13 +115,19 @@ __device__ __noinline__ bool resample_f64(const ResampleArgs& a, int i, int j, i
   if (!ok) atomicOr(&a.ctr->errors, kErrNonFinite);
   if (!ok || t.V == 0.0) return false;
   const double h = (double)a.L.box / a.L.N, inv_gs = 1.0 / a.gs;
+  bool above = false, below = false;
   for (int f = 0; f < 4; ++f) {
     r.d.nx[f] = t.n[f][0];
     r.d.ny[f] = t.n[f][1];
     r.d.d[f] = t.d[f];
     const double big = fmax(fabs(t.n[f][0]), fabs(t.n[f][1]));
     r.d.inz[f] = fabs(t.n[f][2]) > 1e-12 * big ? 1.0 / t.n[f][2] : 0.0;
+    above = above || r.d.inz[f] > 0.0;
+    below = below || r.d.inz[f] < 0.0;
   }
+  // flat in a vertical plane (particles that coincide, but for the rounding of
+  // their place): no face bounds a column in z, and it has no volume but rounding
+  if (!above || !below) return false;
   r.d.q = a.weight == 0 ? a.m_tet / fabs(t.V) : 1.0;
   r.d.qx = i * h;
   r.d.qy = j * h;

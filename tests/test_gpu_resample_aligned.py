@@ -60,3 +60,24 @@ def test_mass_with_an_axis_at_rest(R, N, n, at_rest, half):
 
     here, right, left = planes(0.0), planes(1e-5), planes(-1e-5)
     assert np.all(np.minimum(np.abs(here - right), np.abs(here - left)) <= 1e-3 * here)
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("N,n", [(6, 15), (7, 21), (9, 27), (10, 9), (12, 30), (13, 39)])
+def test_particles_that_coincide(R, N, n, axis):
+    """A seventh of a lattice's particles moved onto their neighbours: tetrahedra
+    flat in the vertical planes that columns run along, with volumes of rounding's
+    size. A cell's line crosses the tetrahedra of a few cubes, no more."""
+    p = particles(N, np.zeros((N ** 3, 3)), False)
+    i = np.arange(N ** 3)
+    a, b, c = i % N, (i // N) % N, i // (N * N)
+    onto = i[((a + 2 * b + 3 * c) % 7 == 3) & (np.maximum(a, b) < N - 2) & (c < N - 1)]
+    for q in onto:
+        p[int(q) + (1, N)[axis]] = p[int(q)]
+    R.build_tets(p, N)
+    streams = R.resample(n, weight="streams").cpu().numpy().astype(np.float64) * n
+    R.sync()
+    assert 0.0 <= streams.min() and streams.max() <= 24.0
+    assert 0.9 <= streams.mean() <= 1.1
+    assert bool(torch.isfinite(R.resample(n, weight="density")).all())
+    R.sync()
